@@ -184,6 +184,27 @@ inline void fill_coef(double rho0, double wp, double wm_run, int collision, cons
 template <typename R>
 inline CoefV<R> coef_cast(const CoefV<double>& d) {
   CoefV<R> c;
+  const double wd = L::w(L::Q - 1);  // diagonal weight of D2Q9 and D3Q19
+  c->wp = wp;
+  c->cpt = -c->cp / 3.0;
+  c->cp2 = 0.5 * c->cp;
+  c->cp4 = 0.25 * c->cp;
+  c->cm2 = 0.5 * c->cm;
+  c->cm4 = 0.25 * c->cm;
+  c->wmd = wm_run * wd;
+  for (int a = 0; a < 3; ++a) {
+    c->hF[a] = hg * F[a];
+    c->hF2[a] = 2.0 * hg * F[a];
+    c->fad[a] = 1.5 * wd * F[a] * (2.0 - wm_run);
+  }
+}
+
+// The coefficients of forcing Scheme II: the F_i projection alone, without the
+// symmetric Guo terms.
+inline CoefV<double> coef_projection(CoefV<double> c) {
+  for (int i = 0; i < kQMax; ++i) c.fe[i] = c.fu[i] = 0.0;
+  for (int a = 0; a < 3; ++a) c.hF[a] = c.hF2[a] = 0.0;
+  return c;
   c.rho0 = R(d.rho0);
   c.cp = R(d.cp);
   c.cm = R(d.cm);
@@ -201,6 +222,18 @@ inline CoefV<R> coef_cast(const CoefV<double>& d) {
 
 const Ops* ops_d2q9_f64();
 const Ops* ops_d2q9_f32();
+  c.wp = R(d.wp);
+  c.cpt = R(d.cpt);
+  c.cp2 = R(d.cp2);
+  c.cp4 = R(d.cp4);
+  c.cm2 = R(d.cm2);
+  c.cm4 = R(d.cm4);
+  c.wmd = R(d.wmd);
+  for (int a = 0; a < 3; ++a) {
+    c.hF[a] = R(d.hF[a]);
+    c.hF2[a] = R(d.hF2[a]);
+    c.fad[a] = R(d.fad[a]);
+  }
 const Ops* ops_d2q9_f16();
 const Ops* ops_d2q9_bf16();
 const Ops* ops_d3q19_f64();

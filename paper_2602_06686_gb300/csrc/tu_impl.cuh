@@ -673,9 +673,7 @@ struct TU {
     a.phi = s.phi;
     a.gk = R(0);
     if (MODE == 2) {
-      CoefV<double> c = s.c;  // the F_i projection: no symmetric Guo terms
-      for (int i = 0; i < kQMax; ++i) c.fe[i] = c.fu[i] = 0.0;
-      a.c = coef_cast<R>(c);
+      a.c = coef_cast<R>(coef_projection(s.c));
       a.gk = R(-4.5 * (1.0 - 0.5 * (1.0 - s.c.cp)));
     }
     size_t smem = tma_smem(XT, a.stages);
@@ -886,9 +884,7 @@ struct TU {
     R* phi = static_cast<R*>(s.phi);
     StepArgs<R> a = args(s);
     k_phi<L, S><<<grid, 256, 0, s.stream>>>(a, s.layout, s.parity, phi);
-    CoefV<double> c = s.c;  // the F_i projection: no symmetric Guo terms
-    for (int i = 0; i < kQMax; ++i) c.fe[i] = c.fu[i] = 0.0;
-    a.c = coef_cast<R>(c);
+    a.c = coef_cast<R>(coef_projection(s.c));
     const R gk = R(-4.5 * (1.0 - 0.5 * (1.0 - s.c.cp)));
     if (s.layout == 1)
       k_step_s2_aa<L, COLL, FORCE, S><<<grid, 256, 0, s.stream>>>(a, s.parity, phi, gk);
