@@ -179,11 +179,6 @@ inline void fill_coef(double rho0, double wp, double wm_run, int collision, cons
     c->fu[i] = -3.0 * w * hg;
     c->fa[i] = collision == 1 ? 1.5 * w * eF : 1.5 * w * eF * (2.0 - wm_run);
   }
-}
-
-template <typename R>
-inline CoefV<R> coef_cast(const CoefV<double>& d) {
-  CoefV<R> c;
   const double wd = L::w(L::Q - 1);  // diagonal weight of D2Q9 and D3Q19
   c->wp = wp;
   c->cpt = -c->cp / 3.0;
@@ -205,6 +200,11 @@ inline CoefV<double> coef_projection(CoefV<double> c) {
   for (int i = 0; i < kQMax; ++i) c.fe[i] = c.fu[i] = 0.0;
   for (int a = 0; a < 3; ++a) c.hF[a] = c.hF2[a] = 0.0;
   return c;
+}
+
+template <typename R>
+inline CoefV<R> coef_cast(const CoefV<double>& d) {
+  CoefV<R> c;
   c.rho0 = R(d.rho0);
   c.cp = R(d.cp);
   c.cm = R(d.cm);
@@ -217,11 +217,6 @@ inline CoefV<double> coef_projection(CoefV<double> c) {
     c.fu[i] = R(d.fu[i]);
     c.fa[i] = R(d.fa[i]);
   }
-  return c;
-}
-
-const Ops* ops_d2q9_f64();
-const Ops* ops_d2q9_f32();
   c.wp = R(d.wp);
   c.cpt = R(d.cpt);
   c.cp2 = R(d.cp2);
@@ -234,6 +229,11 @@ const Ops* ops_d2q9_f32();
     c.hF2[a] = R(d.hF2[a]);
     c.fad[a] = R(d.fad[a]);
   }
+  return c;
+}
+
+const Ops* ops_d2q9_f64();
+const Ops* ops_d2q9_f32();
 const Ops* ops_d2q9_f16();
 const Ops* ops_d2q9_bf16();
 const Ops* ops_d3q19_f64();
