@@ -92,7 +92,8 @@ __device__ __forceinline__ void aa_node(const StepArgs<typename S::R>& a, int x,
 }
 
 template <class L, int COLL, class S, int NV, bool MASK>
-__global__ void __launch_bounds__(256) k_step_aa_even(const StepArgs<typename S::R> a) {
+__global__ void __launch_bounds__(256) k_step_aa_even(StepArgs<typename S::R> a) {
+  a.dst = chain_wait(a.dst);
   if constexpr (NV == 1) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -101,7 +102,8 @@ __global__ void __launch_bounds__(256) k_step_aa_even(const StepArgs<typename S:
 }
 
 template <class L, int COLL, class S, int NV, bool MASK>
-__global__ void __launch_bounds__(256) k_step_aa_odd(const StepArgs<typename S::R> a) {
+__global__ void __launch_bounds__(256) k_step_aa_odd(StepArgs<typename S::R> a) {
+  a.dst = chain_wait(a.dst);
   if constexpr (NV == 1) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, ODD ? 1 : 0>::kThreads,
   __syncthreads();
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* buf = static_cast<T*>(a.dst);
+  T* buf = static_cast<T*>(chain_wait(a.dst));
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer

@@ -46,6 +46,20 @@ struct StepArgs {
   unsigned int step;    // index of the step being computed
 };
 
+// Programmatic dependent launch between consecutive update kernels of a stream
+// (launch_chained): the next launch's blocks are placed while this one runs and
+// wait here until it has completed and its writes are visible.  Every thread of
+// a chained kernel calls it before it touches global memory; the pointer passes
+// through, so that no load of it (read-only path included) can move above the
+// wait.  A launch lets its successor start once it has passed its own wait, so
+// at most one launch waits behind a running one.
+template <typename P>
+__device__ __forceinline__ P* chain_wait(P* p) {
+  asm volatile("griddepcontrol.wait;" : "+l"(p)::"memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  return p;
+}
+
 __device__ __forceinline__ unsigned lane_id() {
   unsigned l;
   asm("mov.u32 %0, %%laneid;" : "=r"(l));
@@ -220,7 +234,8 @@ __device__ __forceinline__ void update_chunk(const StepArgs<typename S::R>& a, i
 
 // Grid: x = ceil(nx / (NV * blockDim.x)) chunks-blocks, y = ceil(ny / blockDim.y), z = nz.
 template <class L, int COLL, class S, int NV, bool MASK>
-__global__ void __launch_bounds__(256) k_step_ab(const StepArgs<typename S::R> a) {
+__global__ void __launch_bounds__(256) k_step_ab(StepArgs<typename S::R> a) {
+  a.src = chain_wait(a.src);
   const int lane = threadIdx.x & 31;
   const int x0 = (blockIdx.x * blockDim.x + threadIdx.x) * NV;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;

@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
   __syncthreads();
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const T* __restrict__ src = static_cast<const T*>(a.src);
+  const T* __restrict__ src = static_cast<const T*>(chain_wait(a.src));
   T* __restrict__ dst = static_cast<T*>(a.dst);
 
   if (warp == 0) {
