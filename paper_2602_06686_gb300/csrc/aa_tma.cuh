@@ -239,6 +239,18 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, ODD ? 1 : 0>::kThreads,
     bool act[NPT];
 #pragma unroll
     for (int n = 0; n < NPT; ++n) act[n] = jn[n] < wdt;
+    if constexpr (!ODD) {  // (the odd step's staging counts every warp)
+      // a warp beyond the row's end has no node in this tile: it releases the
+      // stage and spends no arithmetic on it
+      if (__all_sync(0xffffffffu, !act[0])) {
+        if (lane == 0) mbar_arrive(smem_addr(empty + s));
+        if (++s == ST) {
+          s = 0;
+          ++u;
+        }
+        continue;
+      }
+    }
     V g[L::Q];
     if (!anywall && !xwall) {
 #pragma unroll

@@ -555,6 +555,16 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
       bool act[4];
 #pragma unroll
       for (int n = 0; n < 4; ++n) act[n] = j0 + n < wdt;
+      // a warp beyond the row's end has no node in this tile: it releases the
+      // stage and spends no arithmetic on it
+      if (__all_sync(0xffffffffu, !act[0])) {
+        if (lane == 0) mbar_arrive(smem_addr(empty + s));
+        if (++s == ST) {
+          s = 0;
+          ++u;
+        }
+        continue;
+      }
       F2 ga[L::Q], gb[L::Q];
       if (!anywall && !xwall) {
 #pragma unroll
@@ -664,6 +674,18 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
     bool act[NPT];
 #pragma unroll
     for (int n = 0; n < NPT; ++n) act[n] = jn[n] < wdt;
+    if constexpr (MODE != 3) {
+      // a warp beyond the row's end has no node in this tile: it releases the
+      // stage and spends no arithmetic on it
+      if (__all_sync(0xffffffffu, !act[0])) {
+        if (lane == 0) mbar_arrive(smem_addr(empty + s));
+        if (++s == ST) {
+          s = 0;
+          ++u;
+        }
+        continue;
+      }
+    }
     V g[L::Q];
     if (!anywall && !xwall) {
 #pragma unroll
