@@ -92,20 +92,20 @@ __device__ __forceinline__ void aa_node(const StepArgs<typename S::R>& a, int x,
 }
 
 template <class L, int COLL, class S, int NV, bool MASK>
-__global__ void __launch_bounds__(256) k_step_aa_even(StepArgs<typename S::R> a) {
-  a.dst = chain_wait(a.dst);
+__global__ void __launch_bounds__(256) k_step_aa_even(const StepArgs<typename S::R> a) {
+  const int t = chain_wait((int)threadIdx.x);
   if constexpr (NV == 1) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int x = blockIdx.x * blockDim.x + t;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x < a.g.nx && y < a.g.ny) aa_node<L, COLL, S, MASK>(a, x, y, blockIdx.z, 0);
   }
 }
 
 template <class L, int COLL, class S, int NV, bool MASK>
-__global__ void __launch_bounds__(256) k_step_aa_odd(StepArgs<typename S::R> a) {
-  a.dst = chain_wait(a.dst);
+__global__ void __launch_bounds__(256) k_step_aa_odd(const StepArgs<typename S::R> a) {
+  const int t = chain_wait((int)threadIdx.x);
   if constexpr (NV == 1) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int x = blockIdx.x * blockDim.x + t;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x < a.g.nx && y < a.g.ny) aa_node<L, COLL, S, MASK>(a, x, y, blockIdx.z, 1);
   }

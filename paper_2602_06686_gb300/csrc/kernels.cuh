@@ -49,15 +49,24 @@ struct StepArgs {
 // Programmatic dependent launch between consecutive update kernels of a stream
 // (launch_chained): the next launch's blocks are placed while this one runs and
 // wait here until it has completed and its writes are visible.  Every thread of
-// a chained kernel calls it before it touches global memory; the pointer passes
-// through, so that no load of it (read-only path included) can move above the
-// wait.  A launch lets its successor start once it has passed its own wait, so
+// a chained kernel calls it before it touches global memory.  A value that every
+// address depends on passes through, so that no load (read-only path included)
+// can move above the wait: the base pointer in the pipelined kernels, which
+// hold it in a register anyway, and the node's x in the one-pass kernels, whose
+// base pointers stay kernel parameters (passing the pointer through there costs
+// 4 to 8 registers: D2Q9 FP16 four nodes per thread 64 -> 72, 3 % of a
+// 2250 x 1410 step; FP32 with a mask 6 % of a 2048 x 1024 step).  A launch lets its successor start once it has passed its own wait, so
 // at most one launch waits behind a running one.
 template <typename P>
 __device__ __forceinline__ P* chain_wait(P* p) {
   asm volatile("griddepcontrol.wait;" : "+l"(p)::"memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   return p;
+}
+__device__ __forceinline__ int chain_wait(int x) {
+  asm volatile("griddepcontrol.wait;" : "+r"(x)::"memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  return x;
 }
 
 __device__ __forceinline__ unsigned lane_id() {
@@ -234,10 +243,9 @@ __device__ __forceinline__ void update_chunk(const StepArgs<typename S::R>& a, i
 
 // Grid: x = ceil(nx / (NV * blockDim.x)) chunks-blocks, y = ceil(ny / blockDim.y), z = nz.
 template <class L, int COLL, class S, int NV, bool MASK>
-__global__ void __launch_bounds__(256) k_step_ab(StepArgs<typename S::R> a) {
-  a.src = chain_wait(a.src);
+__global__ void __launch_bounds__(256) k_step_ab(const StepArgs<typename S::R> a) {
   const int lane = threadIdx.x & 31;
-  const int x0 = (blockIdx.x * blockDim.x + threadIdx.x) * NV;
+  const int x0 = chain_wait((int)(blockIdx.x * blockDim.x + threadIdx.x)) * NV;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
   if (y >= a.g.ny) return;  // whole warps (blockDim.x is a multiple of 32)

@@ -62,9 +62,11 @@ struct RowNode {
   int x, y, z;
   long long n;
   bool valid;
-  __device__ __forceinline__ RowNode(const Geo& G) {
+  __device__ __forceinline__ RowNode(const Geo& G) : RowNode(G, threadIdx.x) {}
+  // t: threadIdx.x, in a chained kernel as chain_wait returned it
+  __device__ __forceinline__ RowNode(const Geo& G, int t) {
     const int r = blockIdx.x;
-    x = blockIdx.y * blockDim.x + threadIdx.x;
+    x = blockIdx.y * blockDim.x + t;
     y = r % G.ny;
     z = r / G.ny;
     n = (long long)r * G.nx + x;
@@ -109,13 +111,12 @@ __device__ __forceinline__ void open_fix(int x, int nx, R (&g)[L::Q], R rho0, R 
 // One fused update with the open boundaries (A/B layout, one node per thread,
 // grid of (row, x block) as the helper kernels).
 template <class L, int COLL, class S>
-__global__ void __launch_bounds__(256) k_step_open(StepArgs<typename S::R> a, int fix,
+__global__ void __launch_bounds__(256) k_step_open(const StepArgs<typename S::R> a, int fix,
                                                    typename S::R u_in, typename S::R rho_out) {
   using R = typename S::R;
   using T = typename S::T;
   const Geo& G = a.g;
-  const RowNode q(G);
-  a.src = chain_wait(a.src);
+  const RowNode q(G, chain_wait((int)threadIdx.x));
   if (!q.valid || (a.mask && a.mask[q.n])) return;
   const T* __restrict__ src = static_cast<const T*>(a.src);
   T* __restrict__ dst = static_cast<T*>(a.dst);
@@ -141,13 +142,12 @@ __global__ void __launch_bounds__(256) k_step_open(StepArgs<typename S::R> a, in
 // neighbours are fluid nodes (a periodic axis wraps), one-sided where one is
 // solid or beyond a non-periodic edge, zero where both are.
 template <class L, class S>
-__global__ void __launch_bounds__(256) k_phi(StepArgs<typename S::R> a, int layout,
+__global__ void __launch_bounds__(256) k_phi(const StepArgs<typename S::R> a, int layout,
                                              int parity, typename S::R* phi) {
   using R = typename S::R;
   using T = typename S::T;
   const Geo& G = a.g;
-  const RowNode q(G);
-  a.src = chain_wait(a.src);
+  const RowNode q(G, chain_wait((int)threadIdx.x));
   if (!q.valid || (a.mask && a.mask[q.n])) return;
   const T* __restrict__ src = static_cast<const T*>(a.src);
   R drho = R(0), j[3] = {R(0), R(0), R(0)};
@@ -176,14 +176,13 @@ __global__ void __launch_bounds__(256) k_phi(StepArgs<typename S::R> a, int layo
 //   G_i = gk w_i (sum_a e_ia^2 D_a - (1/3) sum_a D_a),  gk = -(1 - w+/2) / (6 cs^6) = -4.5 (1 - w+/2),
 // i.e. -(1 - w+/2) w_i H2_i:dPhi / (6 cs^6) for the diagonal dPhi = diag(D_a).
 template <class L, int COLL, bool FORCE, class S>
-__global__ void __launch_bounds__(256) k_step_s2(StepArgs<typename S::R> a,
+__global__ void __launch_bounds__(256) k_step_s2(const StepArgs<typename S::R> a,
                                                  const typename S::R* phi,
                                                  typename S::R gk) {
   using R = typename S::R;
   using T = typename S::T;
   const Geo& G = a.g;
-  const RowNode q(G);
-  a.src = chain_wait(a.src);
+  const RowNode q(G, chain_wait((int)threadIdx.x));
   if (!q.valid || (a.mask && a.mask[q.n])) return;
   const T* __restrict__ src = static_cast<const T*>(a.src);
   T* __restrict__ dst = static_cast<T*>(a.dst);
@@ -210,14 +209,13 @@ __global__ void __launch_bounds__(256) k_step_s2(StepArgs<typename S::R> a,
 // The Scheme II update on the AA layout, in place as aa_node: the node reads
 // its slot set through aa_state_slot and writes f*_i + G_i back into it.
 template <class L, int COLL, bool FORCE, class S>
-__global__ void __launch_bounds__(256) k_step_s2_aa(StepArgs<typename S::R> a, int parity,
+__global__ void __launch_bounds__(256) k_step_s2_aa(const StepArgs<typename S::R> a, int parity,
                                                     const typename S::R* phi,
                                                     typename S::R gk) {
   using R = typename S::R;
   using T = typename S::T;
   const Geo& G = a.g;
-  const RowNode q(G);
-  a.dst = chain_wait(a.dst);
+  const RowNode q(G, chain_wait((int)threadIdx.x));
   if (!q.valid || (a.mask && a.mask[q.n])) return;
   T* buf = static_cast<T*>(a.dst);
   R g[L::Q];
