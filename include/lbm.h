@@ -317,7 +317,10 @@ const char* lbm_last_error(void);
 /* Kernel variants (nodes per thread, block shape) available for this context,
  * their names, the selected one, and selection by index.  lbm_set_variant runs
  * every step with the chosen variant; on the AA layout lbm_autotune may choose
- * another for the odd steps (lbm_get_variant reports the even steps' one). */
+ * another for the odd steps (lbm_get_variant reports the even steps' one).
+ * Variants named tma2_* take two steps per launch: lbm_step(n) runs 2 (n / 4) such
+ * launches and the rest of the n steps singly, so that the state is in the same
+ * buffer as after n single steps, and the bits of the state are the same. */
 int lbm_variant_count(const lbm_ctx* ctx, int* n);
 int lbm_variant_name(const lbm_ctx* ctx, int v, char* buf, size_t len);
 int lbm_get_variant(const lbm_ctx* ctx, int* v);

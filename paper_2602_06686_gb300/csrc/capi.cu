@@ -158,10 +158,18 @@ std::vector<Variant> variants_for(const Plan& pl, const Ops* ops, bool masked) {
     for (auto& s : shapes)
       if ((pl.p.ny + s[1] - 1) / s[1] <= 65535) v.push_back(Variant{0, nv, s[0], s[1], 0, 0});
   }
+  // two steps per launch: periodic D2Q9 with 32- or 16-bit storage in the A/B layout
+  if (!masked && pl.p.layout == LBM_LAYOUT_AB && pl.p.periodic[0] && pl.p.periodic[1]) {
+    int sw, ns;
+    for (int X : {512, 256})
+      if (ops->pair_smem(X, 3) > 0 && pair_strips(pl.p.nx, pl.esize, X, &sw, &ns))
+        v.push_back(Variant{2, 0, 0, 0, X, 3});
+  }
   return v;
 }
 
-int default_variant(const Plan& pl, const std::vector<Variant>& vs) {
+// Default of a single step.
+static int default_single(const Plan& pl, const std::vector<Variant>& vs) {
   // the pipelined kernel when available, else the widest vector that keeps the
   // registers of one thread moderate, 256 threads
   for (size_t k = 0; k < vs.size(); ++k)
@@ -177,6 +185,23 @@ int default_variant(const Plan& pl, const std::vector<Variant>& vs) {
     }
   }
   return best;
+}
+
+int default_variant(const Plan& pl, const std::vector<Variant>& vs) {
+  // Two steps per launch where they are available: they beat the fastest
+  // single-step variant on every size measured (us per step, GB300; FP32: 64^2
+  // 2.4 / 3.2, 1024^2 8.6 / 10.7, 2048^2 27 / 48, 4096^2 98 / 183, 64 x 65536 70 / 131;
+  // rows that are no multiple of 16 bytes, which the single-step pipeline does
+  // not take: FP32 1001 x 999 8.8 / 19, FP16 2250 x 1410 27 / 57, 4097 x 4099 139 / 411),
+  // except on large lattices with 16-bit storage and whole 16-byte rows, which
+  // the arithmetic bounds: FP16 64^2 2.6 / 3.2, 1024^2 9.5 / 8.9 (10.3 untuned), 4096^2
+  // 110 / 96 (110 untuned).
+  // Strips of 256 for the rows they hold whole (64 x 65536: 70 against 104 with
+  // 512), else 512 (4096^2: 98 against 108).  A 4-deep ring gains nothing.
+  const bool bound = pl.esize == 2 && pl.p.nx % 8 == 0 && pl.N > (1LL << 21);
+  for (size_t k = 0; k < vs.size(); ++k)
+    if (!bound && vs[k].kind == 2 && vs[k].X == (pl.p.nx <= 256 ? 256 : 512)) return (int)k;
+  return default_single(pl, vs);
 }
 
 }  // namespace lbm
@@ -197,6 +222,7 @@ struct lbm_ctx {
   long long launches = 0;
   std::vector<Variant> vars;
   int var = 0;
+  int var_one = 0;    // variant of a single step where `var` takes two per launch, else var
   int var_odd = -1;   // AA: variant of the odd steps when tuned apart (-1: var)
   int sms = 0;
   OpenBC open{};  // open boundaries of the square-cylinder benchmark (off by default)
@@ -256,6 +282,13 @@ StepLaunch step_of(lbm_ctx* c, const Variant& v) {
   return s;
 }
 
+// The variant that a single step runs with when `var` is selected: `var` itself,
+// or the default of single steps where `var` takes two steps per launch.
+static int single_variant(const Plan& pl, const std::vector<Variant>& vs, int var) {
+  if (vs[var].kind != 2) return var;
+  return default_single(pl, vs);
+}
+
 int ctx_new(const Plan& pl, cudaStream_t st, lbm_ctx** out) {
   lbm_ctx* c = new (std::nothrow) lbm_ctx();
   if (!c) return fail(LBM_ERR_ARG, "out of host memory");
@@ -266,6 +299,7 @@ int ctx_new(const Plan& pl, cudaStream_t st, lbm_ctx** out) {
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   c->vars = variants_for(pl, c->ops, false);
   c->var = default_variant(pl, c->vars);
+  c->var_one = single_variant(c->pl, c->vars, c->var);
   *out = c;
   return LBM_OK;
 }
@@ -281,6 +315,7 @@ int ctx_bind(lbm_ctx* c, void* a, void* b, const uint8_t* mask, void* scratch) {
   c->t = 0;
   c->vars = variants_for(c->pl, c->ops, mask != nullptr);
   c->var = default_variant(c->pl, c->vars);
+  c->var_one = single_variant(c->pl, c->vars, c->var);
   c->var_odd = -1;
   return LBM_OK;
 }
@@ -294,10 +329,23 @@ int reset_flag(lbm_ctx* c) {
 }
 
 int ctx_step(lbm_ctx* c, int n) {
+  if (c->vars[c->var].kind == 2 && c->scheme == 1 && !c->open.on) {
+    // an even number of two-step launches, so that the state ends in the buffer
+    // in which n single steps would leave it
+    for (int p = 2 * (n / 4); p > 0; --p) {
+      cudaError_t e = c->ops->step(step_of(c, c->vars[c->var]));
+      ++c->launches;
+      if (e != cudaSuccess) return fail(LBM_ERR_CUDA, "stream-collide launch", e);
+      c->cur ^= 1;
+      c->t += 2;
+      c->fresh = false;
+      n -= 2;
+    }
+  }
   for (int s = 0; s < n; ++s) {
     const bool odd_own = c->pl.p.layout == LBM_LAYOUT_AA && (c->t & 1) && c->var_odd >= 0 &&
                          c->var_odd < (int)c->vars.size();
-    StepLaunch sl = step_of(c, c->vars[odd_own ? c->var_odd : c->var]);
+    StepLaunch sl = step_of(c, c->vars[odd_own ? c->var_odd : c->var_one]);
     cudaError_t e = c->ops->step(sl);
     c->launches += c->scheme == 2 ? 2 : 1;
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, "stream-collide launch", e);
@@ -321,7 +369,7 @@ void ctx_set_flag(lbm_ctx* c, unsigned int* flag) { c->flag = flag; }
 cudaStream_t ctx_stream(const lbm_ctx* c) { return c->stream; }
 const Ops* ctx_ops(const lbm_ctx* c) { return c->ops; }
 const std::vector<Variant>& ctx_variants(const lbm_ctx* c) { return c->vars; }
-int ctx_variant(const lbm_ctx* c) { return c->var; }
+int ctx_variant(const lbm_ctx* c) { return c->var_one; }
 StepLaunch ctx_step_launch(lbm_ctx* c, const Variant& v) { return step_of(c, v); }
 void ctx_delete(lbm_ctx* c) { delete c; }
 void ctx_add_launches(lbm_ctx* c, long long n) { c->launches += n; }
@@ -710,7 +758,9 @@ int lbm_variant_count(const lbm_ctx* c, int* n) {
 int lbm_variant_name(const lbm_ctx* c, int v, char* buf, size_t len) {
   if (!c || !buf || v < 0 || v >= (int)c->vars.size()) return fail(LBM_ERR_ARG, "bad variant");
   const Variant& x = c->vars[v];
-  if (x.kind == 1 && x.by == 1)
+  if (x.kind == 2)
+    snprintf(buf, len, "tma2_X%d_s%d", x.X, x.stages);
+  else if (x.kind == 1 && x.by == 1)
     snprintf(buf, len, "tma_X%d_s%d_bs", x.X, x.stages);
   else if (x.kind == 1 && x.nv == 4)
     snprintf(buf, len, "tma_X%d_s%d_q", x.X, x.stages);
@@ -732,6 +782,7 @@ int lbm_get_variant(const lbm_ctx* c, int* v) {
 int lbm_set_variant(lbm_ctx* c, int v) {
   if (!c || v < 0 || v >= (int)c->vars.size()) return fail(LBM_ERR_ARG, "bad variant");
   c->var = v;
+  c->var_one = single_variant(c->pl, c->vars, v);
   c->var_odd = -1;
   return LBM_OK;
 }
@@ -742,17 +793,17 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
   const bool aa = c->pl.p.layout == LBM_LAYOUT_AA;
   using Key = std::tuple<int, int, int, int, int, int, int, int, int, int, int, int>;
   static std::mutex mu;
-  static std::map<Key, std::pair<int, int>> cache;  // (variant, AA odd-step variant or -1)
+  // variant, AA odd-step variant or -1, variant of single steps
+  static std::map<Key, std::tuple<int, int, int>> cache;
   const Key key{c->pl.p.lattice, c->pl.p.storage, c->pl.kernel_collision, c->mask != nullptr,
                 c->pl.p.nx,      c->pl.p.ny,      c->pl.p.nz,            c->pl.g.per[0],
                 c->pl.g.per[1],  c->pl.g.per[2],  c->pl.p.layout,        c->scheme};
   if (!times_ms) {
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
-    if (it != cache.end() && it->second.first < (int)c->vars.size() &&
-        it->second.second < (int)c->vars.size()) {
-      c->var = it->second.first;
-      c->var_odd = it->second.second;
+    if (it != cache.end() && std::get<0>(it->second) < (int)c->vars.size() &&
+        std::get<1>(it->second) < (int)c->vars.size() && std::get<2>(it->second) < (int)c->vars.size()) {
+      std::tie(c->var, c->var_odd, c->var_one) = it->second;
       if (chosen) *chosen = c->var;
       return LBM_OK;
     }
@@ -765,9 +816,9 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
     cudaEventDestroy(e0);
     return rc;
   }
-  int best = c->var;
-  float best_ms = 1e30f;
-  const int keep = c->var, keep_odd = c->var_odd;
+  int best = c->var, best_one = c->var_one;
+  float best_ms = 1e30f, best_one_ms = 1e30f;
+  const int keep = c->var, keep_one = c->var_one, keep_odd = c->var_odd;
   // AA: the even and odd steps are different kernels; each gets its fastest
   // variant (timed on steps that really advance the lattice)
   int best_even = c->var, best_odd = c->var;
@@ -778,7 +829,7 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
   for (int v = 0; v < (int)c->vars.size() && rc == LBM_OK; ++v) {
     cudaError_t e = cudaSuccess;
     if (aa) {
-      c->var = v;
+      c->var = c->var_one = v;
       rc = ctx_step(c, (c->t & 1) ? 3 : 2);  // warm up, end on an even step count
       if (rc) break;
       float even_ms = 0.f, odd_ms = 0.f;
@@ -813,8 +864,12 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
       }
       continue;
     }
+    // two steps per launch: not under forcing scheme 2 or open boundaries, where
+    // the steps run singly
+    const bool two = c->vars[v].kind == 2;
+    const int vrun = two && (c->scheme == 2 || c->open.on) ? single_variant(c->pl, c->vars, v) : v;
     {
-      StepLaunch sl = step_of(c, c->vars[v]);  // reads the state, writes the other buffer
+      StepLaunch sl = step_of(c, c->vars[vrun]);  // reads the state, writes the other buffer
       e = c->ops->step(sl);
       c->launches += (1 + reps) * (c->scheme == 2 ? 2 : 1);
       if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
@@ -828,8 +883,12 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
       rc = fail(LBM_ERR_CUDA, "autotune", e);
       break;
     }
-    ms /= reps;
+    ms /= two && vrun == v ? 2 * reps : reps;
     if (times_ms) times_ms[v] = ms;
+    if (!two && ms < best_one_ms) {
+      best_one_ms = ms;
+      best_one = v;
+    }
     if (ms < best_ms) {
       best_ms = ms;
       best = v;
@@ -840,17 +899,19 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
   if (e2) cudaEventDestroy(e2);
   if (rc) {
     c->var = keep;
+    c->var_one = keep_one;
     c->var_odd = keep_odd;
     return rc;
   }
   if (aa) {
-    best = best_even;
+    best = best_one = best_even;
     c->var_odd = best_odd;
   }
   c->var = best;
+  c->var_one = c->vars[best].kind == 2 ? best_one : best;
   {
     std::lock_guard<std::mutex> lk(mu);
-    cache[key] = {best, c->var_odd};
+    cache[key] = std::make_tuple(best, c->var_odd, c->var_one);
   }
   if (chosen) *chosen = best;
   return LBM_OK;

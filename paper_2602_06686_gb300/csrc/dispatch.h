@@ -17,7 +17,8 @@ struct GeoH {
 };
 
 struct Variant {
-  int kind;    // 0: register kernel (one warp row per block row), 1: bulk-copy pipelined kernel
+  int kind;    // 0: register kernel (one warp row per block row), 1: bulk-copy pipelined kernel,
+               // 2: two steps per launch (pair_tma.cuh), X the widest strip
   int nv;      // kind 0: nodes per thread along x; kind 1: 4 for four nodes per consumer
                // thread (16-bit storage, A/B), else 0
   int bx;      // kind 0: threads per block along x (multiple of 32); kind 1: at most this
@@ -135,7 +136,26 @@ struct Ops {
   int (*batch_tma_blocks_per_sm)(int collision, bool force, int X, int stages);
   // shared-memory bytes of the pipelined kernel for a tile width and ring depth (0: unsupported)
   size_t (*tma_smem)(int X, int stages);
+  // the same for the kernel that takes two steps per launch (strip width, ring depth)
+  size_t (*pair_smem)(int X, int stages);
 };
+
+// Strips of the kernel that takes two steps per launch: their width (a multiple
+// of 64, at most X) and number for rows of nx nodes.  The last strip may be narrower,
+// but not below 16 nodes, so that its neighbour's window does not reach
+// past the row's end.  false: no such width (or a row below 32 bytes).
+inline bool pair_strips(int nx, int esize, int X, int* sw, int* nstrips) {
+  if (nx < 32 / esize) return false;
+  const int n = (nx + X - 1) / X;
+  for (int w = ((nx + n - 1) / n + 63) / 64 * 64; w >= 64; w -= 64) {
+    const int k = (nx + w - 1) / w;
+    if (k > 1 && nx - (k - 1) * w < 16) continue;
+    *sw = w;
+    *nstrips = k;
+    return true;
+  }
+  return false;
+}
 
 // Staging buffers of the pipelined AA kernel's odd step: two on D2Q9 (its
 // short collision would otherwise wait for the store warp), one on the 3-D

@@ -8,6 +8,7 @@
 #include "tma.cuh"
 #include "batch_tma.cuh"
 #include "aa_tma.cuh"
+#include "pair_tma.cuh"
 
 namespace lbm {
 
@@ -788,6 +789,65 @@ struct TU {
     return cudaErrorInvalidValue;
   }
 
+  // ---- two steps per launch (kind 2)
+  static constexpr bool kPair = L::Q == 9 && sizeof(T) <= 4;
+  static size_t pair_smem_of(int X, int stages) {
+    return kPair && (X == 256 || X == 512) && stages >= 2 && stages <= 8
+               ? pair_smem((int)sizeof(T), X, stages)
+               : 0;
+  }
+  template <int COLL, bool FORCE, int XT>
+  static cudaError_t go_pair_x(const StepLaunch& s) {
+    PairArgs<R> a;
+    a.g = geo(s.g);
+    a.c = coef_cast<R>(s.c);
+    a.src = s.src;
+    a.dst = s.dst;
+    a.flag = s.flag;
+    a.err = s.err;
+    a.step = s.step;
+    a.stages = s.v.stages;
+    a.timeout_ns = s.wait_ns > 0 ? s.wait_ns : 2000000000LL;
+    a.extra_tx = s.extra_tx;
+    if (!pair_strips(s.g.nx, (int)sizeof(T), XT, &a.sw, &a.nstrips)) return cudaErrorInvalidValue;
+    void (*kern)(PairArgs<R>) = &k_step_pair<L, COLL, S, FORCE, XT>;
+    const size_t smem = pair_smem_of(XT, a.stages);
+    if (smem == 0 || smem > 227 * 1024) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PairShape<XT>::kThreads, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    const int resident = per_sm * (s.sms > 0 ? s.sms : 1);
+    int chunks = resident / a.nstrips;
+    if (chunks > s.g.ny) chunks = s.g.ny;
+    if (chunks < 1) chunks = 1;
+    a.nchunks = chunks;
+    return launch_chained(kern, dim3((unsigned)(a.nstrips * chunks)), dim3(PairShape<XT>::kThreads), smem,
+                          s.stream, a);
+  }
+  template <int COLL>
+  static cudaError_t pair_coll(const StepLaunch& s) {
+    if (s.v.X == 512) return s.force ? go_pair_x<COLL, true, 512>(s) : go_pair_x<COLL, false, 512>(s);
+    if (s.v.X == 256) return s.force ? go_pair_x<COLL, true, 256>(s) : go_pair_x<COLL, false, 256>(s);
+    return cudaErrorInvalidValue;
+  }
+  static cudaError_t step_pair(const StepLaunch& s) {
+    if constexpr (kPair) {
+      if (s.mask != nullptr || s.layout != 0 || !s.g.per[0] || !s.g.per[1]) return cudaErrorInvalidValue;
+      switch (s.collision) {
+        case C_TRT:
+          return pair_coll<C_TRT>(s);
+        case C_TRT_RLB:
+          return pair_coll<C_TRT_RLB>(s);
+        case C_P_TRT:
+          return pair_coll<C_P_TRT>(s);
+      }
+    }
+    return cudaErrorInvalidValue;
+  }
+
   template <int NV>
   static cudaError_t step_nv(const StepLaunch& s) {
     const bool m = s.mask != nullptr;
@@ -930,6 +990,7 @@ struct TU {
     if (s.scheme == 2) return step_s2(s);
     if (s.open.on) return step_open(s);
     if (s.v.kind == 1) return step_tma(s);
+    if (s.v.kind == 2) return step_pair(s);
     switch (s.v.nv) {
       case 1:
         return step_nv<1>(s);
@@ -1136,6 +1197,7 @@ struct TU {
         r.batch_tma_blocks_per_sm = &batch_tma_blocks_per_sm;
       }
       r.tma_smem = &tma_smem;
+      r.pair_smem = &pair_smem_of;
       return r;
     }();
     return &o;
