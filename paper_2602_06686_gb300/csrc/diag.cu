@@ -57,28 +57,25 @@ __global__ void __launch_bounds__(DIAG_THREADS)
   block_store(acc, partials);
 }
 
-// out[k] = sum over blocks of partials[b][k] in block order; the flag slot (6)
-// takes the maximum.
+// out[k] = sum over blocks of partials[b][k], one warp per value: lane l sums
+// blocks l, l + 32, ... and the lanes are added in a fixed tree, so the result is
+// deterministic.  The flag slot (6) takes the maximum.
 __global__ void __launch_bounds__(DIAG_THREADS)
-    k_reduce_partials(const double* partials, int blocks, double* out) {
-  __shared__ double sh[DIAG_THREADS];
-  for (int k = 0; k < NVAL; ++k) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < blocks; b += blockDim.x) {
-      const double v = partials[b * NVAL + k];
-      s = (k == 6) ? fmax(s, v) : s + v;
-    }
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o)
-        sh[threadIdx.x] = (k == 6) ? fmax(sh[threadIdx.x], sh[threadIdx.x + o])
-                                   : sh[threadIdx.x] + sh[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[k] = sh[0];
-    __syncthreads();
+    k_reduce_partials(const double* __restrict__ partials, int blocks, double* out) {
+  static_assert(NVAL * 32 == DIAG_THREADS, "one warp per value");
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = 0.0;
+#pragma unroll 8
+  for (int b = lane; b < blocks; b += 32) {
+    const double v = partials[b * NVAL + k];
+    s = (k == 6) ? fmax(s, v) : s + v;
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double v = __shfl_down_sync(0xffffffffu, s, o);
+    s = (k == 6) ? fmax(s, v) : s + v;
+  }
+  if (lane == 0) out[k] = s;
 }
 
 cudaError_t reduce_partials(const double* partials, int blocks, double* out, cudaStream_t st) {

@@ -119,8 +119,8 @@ struct Ops {
   cudaError_t (*set_pop)(const AuxLaunch&, const double* f);
   cudaError_t (*get_pop)(const AuxLaunch&, double* f);
   cudaError_t (*macros)(const AuxLaunch&, double* rho, double* u);
-  // FP64 diagnostics of the current state: drho and u staged in `fields` in the
-  // arithmetic precision ((1 + D) * N values), block partials [blocks][8]
+  // FP64 diagnostics of the current state: u staged in `fields` in the arithmetic
+  // precision (components 1 .. D of (1 + D) * N values), block partials [blocks][8]
   // (blocks <= rows), the eight sums in out[8] (mass, momentum, kinetic energy,
   // enstrophy, flag, 0)
   cudaError_t (*diag)(const AuxLaunch&, void* fields, double* partials, int blocks, double* out);
