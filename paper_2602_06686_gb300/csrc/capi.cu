@@ -126,7 +126,7 @@ int plan(const lbm_params* p, Plan* out) {
 std::vector<Variant> variants_for(const Plan& pl, const Ops* ops, bool masked) {
   static const int shapes[][2] = {{32, 8}, {64, 4}, {128, 2}, {256, 1}, {32, 4}, {64, 2}, {128, 1}};
   std::vector<Variant> v;
-  // pipelined bulk-copy kernel (A/B or AA): no solid mask, rows a multiple of 16 bytes
+  // pipelined bulk-copy kernel (A/B or AA; masked A/B below): rows a multiple of 16 bytes
   const int H = 16 / pl.esize;
   if (!masked && pl.p.nx % H == 0 && pl.p.nx >= 2 * H) {
     static const int tiles[] = {512, 384, 256, 192, 128};
@@ -150,6 +150,14 @@ std::vector<Variant> variants_for(const Plan& pl, const Ops* ops, bool masked) {
             ops->tma_smem(X, st) <= 200 * 1024)
           v.push_back(Variant{1, 4, 0, 0, X, st});
       }
+  }
+  if (masked && pl.p.layout == LBM_LAYOUT_AB && pl.p.nx % H == 0 && pl.p.nx >= 2 * H) {
+    for (int st : {4, 3, 2}) {
+      const size_t smem = ops->tma_smem(ops->mask_tile, st);
+      if (smem == 0 || smem > 200 * 1024) continue;
+      v.push_back(Variant{1, 0, 0, 0, ops->mask_tile, st});
+      v.push_back(Variant{1, 0, 2, 0, ops->mask_tile, st});
+    }
   }
   for (int k = 0; k < ops->n_nv; ++k) {
     const int nv = ops->nvs[k];

@@ -136,6 +136,7 @@ struct Ops {
   int (*batch_tma_blocks_per_sm)(int collision, bool force, int X, int stages);
   // shared-memory bytes of the pipelined kernel for a tile width and ring depth (0: unsupported)
   size_t (*tma_smem)(int X, int stages);
+  int mask_tile;  // its tile width on lattices with a solid mask (A/B)
   // the same for the kernel that takes two steps per launch (strip width, ring depth)
   size_t (*pair_smem)(int X, int stages);
 };

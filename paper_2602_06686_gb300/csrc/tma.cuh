@@ -21,8 +21,10 @@
 //
 // Rows whose source lies beyond a non-periodic wall (halfway bounce-back) are
 // replaced by the node's own row of the opposite plane; x-walls read the
-// opposite plane's own value from HBM (rare, per node).  Masked lattices use
-// the register kernel.
+// opposite plane's own value from HBM (rare, per node).  Masked lattices
+// (MODE 5) look at the mask around a warp's nodes while the stage's copy is in
+// flight; only a warp with a solid node in reach takes the general gather, where
+// a solid source is the node's own opposite value, read from HBM.
 //
 // Every mbarrier wait is bounded by %globaltimer: on time-out the block sets
 // an error word, lets its issued copies land, and returns.
@@ -80,6 +82,7 @@ struct TmaArgs {
   int extra_tx;  // test hook: extra bytes every stage waits for (never delivered)
   void* phi;     // MODE 1 / 2: rho u_a^3, [D][nx * ny * nz] (dense node index), precision R
   R gk;          // MODE 2: -(1 - w+/2) / (6 cs^6)
+  const uint8_t* mask;  // MODE 5: solid nodes, dense [z][y][x]
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -308,6 +311,52 @@ __device__ __forceinline__ R phi_grad(const Geo& G, const uint8_t* mask, const R
   if (okp) return p[np] - p[n];
   if (okm) return p[n] - p[nm];
   return R(0);
+}
+
+// MODE 5 (solid mask): is any node of the neighbourhoods of the warp's 32
+// consecutive nodes solid?  x: this lane's node.  Each lane looks at its column of
+// the 3^(D-1) neighbour rows and the outer lanes at the columns beside the
+// warp's; out-of-range columns are clamped to the row (an extra look can only send
+// the warp down the general path).
+template <class L>
+__device__ __forceinline__ bool mask_near(const Geo& G, const uint8_t* __restrict__ mask, int x, int y,
+                                          int z, int lane) {
+  unsigned any = 0u;
+  const int xl = x == 0 ? G.nx - 1 : x - 1, xr = x >= G.nx - 1 ? 0 : x + 1;
+  const int xc = min(x, G.nx - 1), xs = lane == 0 ? xl : (lane == 31 ? min(xr, G.nx - 1) : xc);
+#pragma unroll
+  for (int dz = (L::D == 3 ? -1 : 0); dz <= (L::D == 3 ? 1 : 0); ++dz) {
+    int zz = z + dz;
+    zz = zz < 0 ? G.nz - 1 : (zz >= G.nz ? 0 : zz);
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy) {
+      int yy = y + dy;
+      yy = yy < 0 ? G.ny - 1 : (yy >= G.ny ? 0 : yy);
+      const uint8_t* row = mask + ((long long)zz * G.ny + yy) * G.nx;
+      any |= row[xc];
+      if (lane == 0 || lane == 31) any |= row[xs];
+    }
+  }
+  return any != 0u;
+}
+
+// Is the node (x - ex, y - ey, z - ez) solid (periodic axes wrap; beyond a
+// non-periodic edge there is no node)?
+__device__ __forceinline__ bool mask_source(const Geo& G, const uint8_t* __restrict__ mask, int x, int y,
+                                            int z) {
+  if (x < 0 || x >= G.nx) {
+    if (!G.per[0]) return false;
+    x = x < 0 ? x + G.nx : x - G.nx;
+  }
+  if (y < 0 || y >= G.ny) {
+    if (!G.per[1]) return false;
+    y = y < 0 ? y + G.ny : y - G.ny;
+  }
+  if (z < 0 || z >= G.nz) {
+    if (!G.per[2]) return false;
+    z = z < 0 ? z + G.nz : z - G.nz;
+  }
+  return mask[((long long)z * G.ny + y) * G.nx + x] != 0;
 }
 
 // Resident blocks per SM the register allocation is asked to allow: 4 for
@@ -659,10 +708,17 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
   uint32_t u = 0;
   int kt = 0;  // MODE 3: tiles done by this block
   for (; w.more(); w.next()) {
-    if (!mbar_wait_warp(smem_addr(full + s), u & 1u, abort_flag, a.err, a.timeout_ns)) break;
     const int y = w.y, z = w.z;
     const int x0 = w.tx * XT;
     const int wdt = min(XT, G.nx - x0);
+    bool near = false;  // MODE 5: a solid node is in reach of this warp's nodes
+    if constexpr (MODE == 5) {
+      // before the wait for the stage, so that the mask's latency overlaps the copy's
+      near = mask_near<L>(G, a.mask, x0 + jn[0], y, z, ADJ ? 0 : lane);
+      if (PACK) near |= mask_near<L>(G, a.mask, x0 + jn[NPT - 1], y, z, ADJ ? 31 : lane);
+      near = __any_sync(0xffffffffu, near);
+    }
+    if (!mbar_wait_warp(smem_addr(full + s), u & 1u, abort_flag, a.err, a.timeout_ns)) break;
     const T* st = reinterpret_cast<const T*>(ringb + s * stage_bytes);
     const long long own = ((long long)z * G.ny + y) * G.pitch;
     // tile-uniform: does any plane's source row lie beyond a wall (|e| <= 1, so
@@ -686,8 +742,15 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
         continue;
       }
     }
+    if constexpr (MODE == 5) {
+      if (near) {
+#pragma unroll
+        for (int n = 0; n < NPT; ++n)
+          act[n] = act[n] && a.mask[((long long)z * G.ny + y) * G.nx + x0 + jn[n]] == 0;
+      }
+    }
     V g[L::Q];
-    if (!anywall && !xwall) {
+    if (!anywall && !xwall && !near) {
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) {
         const T* slot = st + i * SLOT + HT - L::cx(i);
@@ -719,7 +782,10 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
         for (int n = 0; n < NPT; ++n) {
           const int j = jn[n];
           const int x = x0 + j;
-          if (wallrow) {
+          if (MODE == 5 && !wallrow && near && act[n] &&
+              mask_source(G, a.mask, x - ex, y - L::cy(i), z - L::cz(i))) {
+            v[n] = S::dec(src[L::opp(i) * G.plane + own + x]);  // bounce-back at a solid node
+          } else if (wallrow) {
             v[n] = S::dec(slot[j]);
           } else if (!G.per[0] && ((ex == 1 && x == 0) || (ex == -1 && x == G.nx - 1))) {
             v[n] = act[n] ? S::dec(src[L::opp(i) * G.plane + own + x]) : R(0);
@@ -848,7 +914,7 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
       continue;
     }
     T* op = dst + own + x0;
-    if (wdt == XT) {
+    if (wdt == XT && !near) {
       // a full tile: every node is active, the stores need no per-plane test
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) {
