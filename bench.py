@@ -42,11 +42,12 @@ BYTES_PER_NODE = {("D2Q9", "F64"): 144, ("D2Q9", "F32"): 72, ("D2Q9", "F16"): 36
                   ("D3Q27", "F32"): 216, ("D3Q27", "F16"): 108, ("D3Q27", "BF16"): 108}
 PROFILE = os.path.join(ROOT, "profiles", "stream_collide_d2q9_f32_4096.md")
 # FP64 instructions (DADD + DMUL + DFMA) per node update of the FP64 update, by
-# lattice and collision: ncu counts on D3Q19 128^3 and D2Q9 2048x1024
-# (profiles/stream_collide_d3q19_f64_128.md).  With GB300's 2 FP64 lanes per
-# SM they give the FP64-pipe roofline of the FP64 runs.
-FP64_INSTR_PER_NODE = {("D3Q19", "P_TRT"): 242, ("D3Q19", "TRT_RLB"): 301, ("D3Q19", "TRT"): 192,
-                       ("D2Q9", "P_TRT"): 103, ("D2Q9", "TRT_RLB"): 129, ("D2Q9", "TRT"): 93}
+# lattice and collision.  TRT-RLB: ncu counts on D3Q19 128^3 and D2Q9 2048x1024
+# (profiles/stream_collide_d3q19_f64_128.md).  P-TRT and TRT: counted from the
+# moment-space form in collide_v.cuh, with 7 for the reciprocal.  With GB300's 2
+# FP64 lanes per SM they give the FP64-pipe roofline of the FP64 runs.
+FP64_INSTR_PER_NODE = {("D3Q19", "P_TRT"): 162, ("D3Q19", "TRT_RLB"): 301, ("D3Q19", "TRT"): 166,
+                       ("D2Q9", "P_TRT"): 80, ("D2Q9", "TRT_RLB"): 129, ("D2Q9", "TRT"): 82}
 FP64_LANES_PER_SM = 2
 
 
@@ -66,7 +67,7 @@ EXTRA_LEGEND = ("d2q9_*: double shear 4096^2 Re=1e5 1/tau-=1.6; d3q19_*/d3q27_*:
 
 # Device code of the pipelined fused kernel: the committed ncu counters of the
 # headline kernel are used only while these files are unchanged.
-KERNEL_SOURCES = ("tma.cuh", "collide_v.cuh", "storage.cuh", "lattice.cuh", "kernels.cuh")
+KERNEL_SOURCES = ("pair_tma.cuh", "tma.cuh", "collide_v.cuh", "storage.cuh", "lattice.cuh", "kernels.cuh")
 
 
 def csrc_hash() -> str:
@@ -361,6 +362,12 @@ def scheme2_bytes_per_node(lat: str, storage: str) -> int:
     return 3 * BYTES_PER_NODE[(lat, storage)] // 2 + 2 * D * r
 
 
+def step_bytes(lat: str, storage: str, variant: str) -> int:
+    """HBM bytes per node update: a variant that takes two steps per launch
+    (tma2_*) reads and writes the state once for both."""
+    return BYTES_PER_NODE[(lat, storage)] // (2 if variant.startswith("tma2") else 1)
+
+
 def secondary(lat: str, n: int, storage: str, kind: str, peak: float, collision="P_TRT",
               layout: str = "AB", scheme: int = 1):
     """MLUPS and roofline fraction of another workload (kernel-only, few steps):
@@ -374,9 +381,10 @@ def secondary(lat: str, n: int, storage: str, kind: str, peak: float, collision=
         g.set_forcing_scheme(2)
     g.autotune(reps=3, report=False)
     reps = 1 if storage == "F64" and lat != "D2Q9" else 3
-    dt = time_kernel(g, 10, reps)
+    dt = time_kernel(g, 12, reps)  # a multiple of 4: all steps in pairs where they pair
     N = g.N
-    bpn = BYTES_PER_NODE[(lat, storage)] if scheme == 1 else scheme2_bytes_per_node(lat, storage)
+    bpn = (step_bytes(lat, storage, g.variants()[g.variant]) if scheme == 1
+           else scheme2_bytes_per_node(lat, storage))
     gbs = bpn * N / dt / 1e9
     out = {"mlups": N / dt / 1e6, "frac": gbs / peak, "v": g.variants()[g.variant]}
     if storage == "F64" and (lat, collision) in FP64_INSTR_PER_NODE:
@@ -1074,10 +1082,10 @@ def run_ours(args):
     g.macros_host_ptr(rho_o.data_ptr(), u_o.data_ptr())
     t_d2h = time.perf_counter() - t0
 
-    bpn = BYTES_PER_NODE[("D2Q9", "F32")]
+    bpn = step_bytes("D2Q9", "F32", variant)
     achieved = bpn * N / kernel_s / 1e9
     khash = csrc_hash()
-    ceiling = copy_ceiling_at(bpn * N // 2) if rank == 0 else None
+    ceiling = copy_ceiling_at(BYTES_PER_NODE[("D2Q9", "F32")] * N // 2) if rank == 0 else None
     extra = {}
     if rank == 0 and not args.no_extra:
         del g
