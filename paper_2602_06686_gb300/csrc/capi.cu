@@ -178,6 +178,47 @@ std::vector<Variant> variants_for(const Plan& pl, const Ops* ops, bool masked) {
 
 // Default of a single step.
 static int default_single(const Plan& pl, const std::vector<Variant>& vs) {
+  // 16-bit storage, A/B: four nodes per thread (D2Q9 2048^2 27 us a step against 31
+  // with two, 4096^2 96 / 111; D3Q19 256^3 273 / 504, 96^3 38 / 70).
+  const bool aa = pl.p.layout == LBM_LAYOUT_AA;
+  const int quad = pl.esize == 2 && !aa ? 4 : 0;
+  if (pl.Q == 9 && quad)
+    for (size_t k = 0; k < vs.size(); ++k)
+      if (vs[k].kind == 1 && vs[k].nv == 4 && vs[k].X == 512 && vs[k].stages == 2) return (int)k;
+  if (pl.Q > 9 && (!aa || pl.esize == 4)) {  // (AA measured in FP32 only)
+    // Three dimensions: the shallowest ring, since a deep one of 19 or 27 planes
+    // leaves an SM one block (us a step, GB300, depth 2 against 512 or 384 wide and 4
+    // deep: D3Q19 FP32 128^3 90 / 227, 256^3 415 / 943, D3Q27 FP32 192^3 260 / 665, D3Q19
+    // FP64 96^3 288 / 344), and the width that pads a row least; of equal ones
+    // the narrower, in FP64 the wider (D3Q19 FP32 256^3: 256 415, 512 574; FP64: 256 5107,
+    // 128 5159).
+    int best = -1, best_pad = 0;
+    for (int nv = quad; best < 0; nv = 0) {
+      for (size_t k = 0; k < vs.size(); ++k) {
+        const Variant& v = vs[k];
+        if (v.kind != 1 || v.bx != 0 || v.by != 0 || v.nv != nv || v.stages != 2) continue;
+        const int pad = (pl.p.nx + v.X - 1) / v.X * v.X;
+        const bool better = best < 0 || pad < best_pad ||
+                            (pad == best_pad && (pl.esize == 8 ? v.X > vs[best].X : v.X < vs[best].X));
+        if (better) {
+          best = (int)k;
+          best_pad = pad;
+        }
+      }
+      if (nv == 0) break;
+    }
+    // Rows that fill too little of a tile are better off in the register kernel
+    // (D3Q19 FP32 64^3 14.5 us against 23.5, 32^3 5.5 / 8.5, 128^3 109 / 90; AA 160^3, a tile of
+    // 256: 173 / 192; FP16 96^3 49 / 38).  FP64 is bound by its pipe either way.
+    const bool narrow = pl.esize == 8 ? false
+                        : aa          ? 3 * pl.p.nx < 2 * best_pad
+                        : quad        ? pl.p.nx < 96
+                                      : pl.p.nx < 128;
+    if (best >= 0 && !narrow) return best;
+    if (best >= 0)
+      for (size_t k = 0; k < vs.size(); ++k)
+        if (vs[k].kind == 0 && vs[k].nv == 1 && vs[k].bx == 32 && vs[k].by == 8) return (int)k;
+  }
   // the pipelined kernel when available, else the widest vector that keeps the
   // registers of one thread moderate, 256 threads
   for (size_t k = 0; k < vs.size(); ++k)
@@ -202,11 +243,10 @@ int default_variant(const Plan& pl, const std::vector<Variant>& vs) {
   // rows that are no multiple of 16 bytes, which the single-step pipeline does
   // not take: FP32 1001 x 999 8.8 / 19, FP16 2250 x 1410 27 / 57, 4097 x 4099 139 / 411),
   // except on large lattices with 16-bit storage and whole 16-byte rows, which
-  // the arithmetic bounds: FP16 64^2 2.6 / 3.2, 1024^2 9.5 / 8.9 (10.3 untuned), 4096^2
-  // 110 / 96 (110 untuned).
+  // the arithmetic bounds: FP16 64^2 2.6 / 3.2, 1024^2 9.5 / 8.9, 4096^2 110 / 96.
   // Strips of 256 for the rows they hold whole (64 x 65536: 70 against 104 with
   // 512), else 512 (4096^2: 98 against 108).  A 4-deep ring gains nothing.
-  const bool bound = pl.esize == 2 && pl.p.nx % 8 == 0 && pl.N > (1LL << 21);
+  const bool bound = pl.esize == 2 && pl.p.nx % 8 == 0 && pl.N >= (1LL << 20);
   for (size_t k = 0; k < vs.size(); ++k)
     if (!bound && vs[k].kind == 2 && vs[k].X == (pl.p.nx <= 256 ? 256 : 512)) return (int)k;
   return default_single(pl, vs);
