@@ -100,7 +100,10 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, ODD ? 1 : 0>::kThreads,
   __syncthreads();
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* buf = static_cast<T*>(chain_wait(a.dst));
+  // the buffer stays a kernel parameter (global loads and stores, not generic ones);
+  // none of its plain accesses can move above the wait
+  chain_wait((int)threadIdx.x);
+  T* buf = static_cast<T*>(a.dst);
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
