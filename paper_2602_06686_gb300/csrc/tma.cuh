@@ -47,6 +47,7 @@
 #include "collide_v.cuh"
 #include "dispatch.h"
 #include "kernels.cuh"
+#include "mask_look.cuh"
 #include "storage.cuh"
 
 namespace lbm {
@@ -316,14 +317,13 @@ __device__ __forceinline__ R phi_grad(const Geo& G, const uint8_t* mask, const R
 // MODE 5 (solid mask): is any node of the neighbourhoods of the warp's 32
 // consecutive nodes solid?  x: this lane's node.  Each lane looks at its column of
 // the 3^(D-1) neighbour rows and the outer lanes at the columns beside the
-// warp's; out-of-range columns are clamped to the row (an extra look can only send
-// the warp down the general path).
+// warp's (mask_column and mask_column_beside keep every column inside the row; an
+// extra look can only send the warp down the general path).
 template <class L>
 __device__ __forceinline__ bool mask_near(const Geo& G, const uint8_t* __restrict__ mask, int x, int y,
                                           int z, int lane) {
   unsigned any = 0u;
-  const int xl = x == 0 ? G.nx - 1 : x - 1, xr = x >= G.nx - 1 ? 0 : x + 1;
-  const int xc = min(x, G.nx - 1), xs = lane == 0 ? xl : (lane == 31 ? min(xr, G.nx - 1) : xc);
+  const int xc = mask_column(x, G.nx), xs = mask_column_beside(x, G.nx, lane);
 #pragma unroll
   for (int dz = (L::D == 3 ? -1 : 0); dz <= (L::D == 3 ? 1 : 0); ++dz) {
     int zz = z + dz;
@@ -713,10 +713,13 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
     const int wdt = min(XT, G.nx - x0);
     bool near = false;  // MODE 5: a solid node is in reach of this warp's nodes
     if constexpr (MODE == 5) {
-      // before the wait for the stage, so that the mask's latency overlaps the copy's
-      near = mask_near<L>(G, a.mask, x0 + jn[0], y, z, ADJ ? 0 : lane);
-      if (PACK) near |= mask_near<L>(G, a.mask, x0 + jn[NPT - 1], y, z, ADJ ? 31 : lane);
-      near = __any_sync(0xffffffffu, near);
+      // before the wait for the stage, so that the mask's latency overlaps the copy's;
+      // a warp beyond the row's end has no node to look around
+      if (__any_sync(0xffffffffu, jn[0] < wdt)) {
+        near = mask_near<L>(G, a.mask, x0 + jn[0], y, z, ADJ ? 0 : lane);
+        if (PACK) near |= mask_near<L>(G, a.mask, x0 + jn[NPT - 1], y, z, ADJ ? 31 : lane);
+        near = __any_sync(0xffffffffu, near);
+      }
     }
     if (!mbar_wait_warp(smem_addr(full + s), u & 1u, abort_flag, a.err, a.timeout_ns)) break;
     const T* st = reinterpret_cast<const T*>(ringb + s * stage_bytes);
