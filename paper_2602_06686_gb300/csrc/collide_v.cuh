@@ -182,7 +182,7 @@ struct CoefV {
   S cm2, cm4;      // (1 - w-) / 2, / 4
   S wmd;           // w- times the diagonal weight
   S hF[3], hF2[3]; // (1 - w+/2) F and twice that
-  S fad[3];        // antisymmetric force content of a diagonal, per axis
+  S fax[3], fad[3];  // antisymmetric force content of an axial and of a diagonal velocity, per axis
 };
 
 // ---- ghost tables (integer values and s_k^2 / N_k) ------------------------
@@ -381,7 +381,7 @@ __device__ __forceinline__ unsigned collide_planes(V (&g)[L::Q],
     if (kTrt) sym = A::fma(A::c(c.cp2), s[a], sym);
     // the axial weight is w1 = (w1 / w2) w2
     V anti = A::fma(A::c(c.cm2), d[a], A::mul(q[a], A::mul(K[a], A::c(w1 / w2))));
-    if (FORCE) anti = A::add(anti, A::c(c.fa[ip(a)]));
+    if (FORCE) anti = A::add(anti, A::c(c.fax[a]));
     g[ip(a)] = A::add(sym, anti);
     g[im(a)] = A::sub(sym, anti);
   }
