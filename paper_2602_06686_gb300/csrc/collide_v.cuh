@@ -285,6 +285,10 @@ __device__ __forceinline__ V wden_div(V x, int den) {
 //    axis: (e.m)(3 + 4.5 ((e.u)^2 - u^2)) on (+,+) and (+,-) is A +- B with
 //    A = m_a (3 + 4.5 (u_a^2 + 3 u_b^2 - u^2)) and B with a, b exchanged.
 // The Guo source is second order as well: T_ab += (1 - w+/2)(u_a F_b + u_b F_a).
+// The antisymmetric force content enters with the equilibrium's product in one fma: added
+// to the finished sum it costs one more rounding, at the size of the populations
+// and alike on every node of a uniform stream, which compounds (D3Q19, w- = 0.25,
+// 200 steps of a forced vortex: velocity error 8.4e-15 against 2.1e-15; pair by pair 5.8e-15).
 template <class L, int COLL, bool FORCE, typename V>
 __device__ __forceinline__ unsigned collide_planes(V (&g)[L::Q],
                                                    const CoefV<typename Ar<V>::S>& c) {
@@ -380,8 +384,9 @@ __device__ __forceinline__ unsigned collide_planes(V (&g)[L::Q],
     V sym = A::fma(A::c(4.5 * w1), X[a], base1);
     if (kTrt) sym = A::fma(A::c(c.cp2), s[a], sym);
     // the axial weight is w1 = (w1 / w2) w2
-    V anti = A::fma(A::c(c.cm2), d[a], A::mul(q[a], A::mul(K[a], A::c(w1 / w2))));
-    if (FORCE) anti = A::add(anti, A::c(c.fax[a]));
+    const V ka = A::mul(K[a], A::c(w1 / w2));
+    const V eq = FORCE ? A::fma(q[a], ka, A::c(c.fax[a])) : A::mul(q[a], ka);
+    const V anti = A::fma(A::c(c.cm2), d[a], eq);
     g[ip(a)] = A::add(sym, anti);
     g[im(a)] = A::sub(sym, anti);
   }
@@ -394,12 +399,11 @@ __device__ __forceinline__ unsigned collide_planes(V (&g)[L::Q],
       sd = A::fma(A::c(c.cp4), P[k], sd);
       so = A::fma(A::c(c.cp4), Pm[k], so);
     }
-    V aa = A::fma(A::c(c.cm4), Dp[k], A::mul(q[a], A::fma(uu[b], A::c(13.5), K[a])));
-    V ab = A::fma(A::c(c.cm4), Dm[k], A::mul(q[b], A::fma(uu[a], A::c(13.5), K[b])));
-    if (FORCE) {
-      aa = A::add(aa, A::c(c.fad[a]));
-      ab = A::add(ab, A::c(c.fad[b]));
-    }
+    const V ka = A::fma(uu[b], A::c(13.5), K[a]), kb = A::fma(uu[a], A::c(13.5), K[b]);
+    const V qa = FORCE ? A::fma(q[a], ka, A::c(c.fad[a])) : A::mul(q[a], ka);
+    const V qb = FORCE ? A::fma(q[b], kb, A::c(c.fad[b])) : A::mul(q[b], kb);
+    const V aa = A::fma(A::c(c.cm4), Dp[k], qa);
+    const V ab = A::fma(A::c(c.cm4), Dm[k], qb);
     const V e1 = A::add(sd, so), e2 = A::sub(sd, so);
     const V a1 = A::add(aa, ab), a2 = A::sub(aa, ab);
     g[ipp(k)] = A::add(e1, a1);
