@@ -937,11 +937,15 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
       if constexpr (ADJ) {
-        // op + jn[0] is 4-byte aligned (16-byte row pitch, even x0 + jn[0])
-        if (act[NPT - 1]) {
+        // op + jn[0] is 4-byte aligned (16-byte row pitch, even x0 + jn[0]); beside a
+        // solid node (MODE 5) either node of the pair may be the one to store, and the
+        // other's slot is not written
+        if (MODE == 5 ? act[0] && act[NPT - 1] : act[NPT - 1]) {
           *reinterpret_cast<uint32_t*>(op + jn[0]) = S::enc2(g[i].x, g[i].y);
         } else if (act[0]) {
           op[jn[0]] = S::enc(g[i].x);
+        } else if (MODE == 5 && act[NPT - 1]) {
+          op[jn[NPT - 1]] = S::enc(g[i].y);
         }
       } else if constexpr (PACK) {
         if (act[0]) op[jn[0]] = S::enc(g[i].x);
