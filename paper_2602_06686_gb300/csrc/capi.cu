@@ -6,6 +6,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <array>
 #include <map>
 #include <mutex>
 #include <new>
@@ -839,13 +840,16 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
   CHECK_CTX(c);
   if (reps < 1) reps = 1;
   const bool aa = c->pl.p.layout == LBM_LAYOUT_AA;
-  using Key = std::tuple<int, int, int, int, int, int, int, int, int, int, int, int>;
+  // Everything that a candidate's kernel or time depends on.  With open boundaries all of them
+  // run the same kernel, and with a force another instantiation.
+  using Key = std::array<int, 15>;
   static std::mutex mu;
   // variant, AA odd-step variant or -1, variant of single steps
   static std::map<Key, std::tuple<int, int, int>> cache;
   const Key key{c->pl.p.lattice, c->pl.p.storage, c->pl.kernel_collision, c->mask != nullptr,
                 c->pl.p.nx,      c->pl.p.ny,      c->pl.p.nz,            c->pl.g.per[0],
-                c->pl.g.per[1],  c->pl.g.per[2],  c->pl.p.layout,        c->scheme};
+                c->pl.g.per[1],  c->pl.g.per[2],  c->pl.p.layout,        c->scheme,
+                c->open.on,      c->pl.force,     c->device};
   if (!times_ms) {
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
