@@ -8,6 +8,7 @@
 #include "tma.cuh"
 #include "batch_tma.cuh"
 #include "aa_tma.cuh"
+#include "launch_table.h"
 #include "pair_tma.cuh"
 
 namespace lbm {
@@ -600,6 +601,21 @@ inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
 
+// Resident blocks per SM of a kernel with `smem` bytes of dynamic shared memory on the
+// current device, the opt-in to them included (asked for once per device and depth).
+template <typename... P>
+inline cudaError_t resident_blocks(LaunchTable& table, void (*kern)(P...), int threads, size_t smem,
+                                   int depth, int* per_sm) {
+  int device = 0;
+  const cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  return table.get(
+      device, depth,
+      [&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); },
+      [&](int* n) { return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kern, threads, smem); },
+      per_sm);
+}
+
 template <class L, class S>
 struct TU {
   using R = typename S::R;
@@ -723,22 +739,11 @@ struct TU {
       if (kind == 2 || kind == 3) threads = TmaShape<XT, kPack, 1>::kThreads;
       if (kind == 4) threads = TmaShape<XT, kPack, 0, kPack && sizeof(T) == 2 ? 4 : 0>::kThreads;
     }
-    // per instantiation and kind: the shared-memory opt-in (once) and the
-    // resident blocks per SM for each ring depth (cached)
-    static bool attr_set[5] = {false, false, false, false, false};
-    static int per_sm_cache[5][9] = {};
-    if (!attr_set[kind]) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      if (e != cudaSuccess) return e;
-      attr_set[kind] = true;
-    }
-    int per_sm = per_sm_cache[kind][a.stages];
-    if (per_sm == 0) {
-      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-      if (e != cudaSuccess) return e;
-      if (per_sm < 1) return cudaErrorInvalidConfiguration;
-      per_sm_cache[kind][a.stages] = per_sm;
-    }
+    // one table per instantiation and kind
+    static LaunchTable tables[5];
+    int per_sm = 0;
+    cudaError_t e = resident_blocks(tables[kind], kern, threads, smem, a.stages, &per_sm);
+    if (e != cudaSuccess) return e;
     const int resident = s.v.bx > 0 && s.v.bx < per_sm ? s.v.bx : per_sm;
     long long blocks = (long long)resident * (s.sms > 0 ? s.sms : 1);
     if (blocks > a.ntiles) blocks = a.ntiles;
@@ -819,12 +824,10 @@ struct TU {
     void (*kern)(PairArgs<R>) = &k_step_pair<L, COLL, S, FORCE, XT>;
     const size_t smem = pair_smem_of(XT, a.stages);
     if (smem == 0 || smem > 227 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e != cudaSuccess) return e;
+    static LaunchTable table;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PairShape<XT>::kThreads, smem);
+    cudaError_t e = resident_blocks(table, kern, PairShape<XT>::kThreads, smem, a.stages, &per_sm);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int resident = per_sm * (s.sms > 0 ? s.sms : 1);
     int chunks = resident / a.nstrips;
     if (chunks > s.g.ny) chunks = s.g.ny;
