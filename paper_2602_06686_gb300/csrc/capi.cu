@@ -177,8 +177,46 @@ std::vector<Variant> variants_for(const Plan& pl, const Ops* ops, bool masked) {
   return v;
 }
 
+// Register kernel: the widest vector of at most max_nv nodes that keeps the
+// registers of one thread moderate, 256 threads.
+static int default_register(const Plan& pl, const std::vector<Variant>& vs, int max_nv) {
+  const int budget = pl.Q == 9 ? 16 : 8;  // bytes per plane per thread
+  int best = 0, best_nv = 0;
+  for (size_t k = 0; k < vs.size(); ++k) {
+    const Variant& v = vs[k];
+    if (v.kind != 0 || v.nv > max_nv || v.nv * pl.esize > budget || v.bx * v.by != 256) continue;
+    if (v.nv > best_nv || (v.nv == best_nv && v.bx == 64)) {
+      best = (int)k;
+      best_nv = v.nv;
+    }
+  }
+  return best;
+}
+
 // Default of a single step.
-static int default_single(const Plan& pl, const std::vector<Variant>& vs) {
+static int default_single(const Plan& pl, const std::vector<Variant>& vs, bool masked) {
+  if (masked && pl.p.layout == LBM_LAYOUT_AB) {
+    // The pipelined update passes around a few bodies at the copy's pace, but a warp with a
+    // solid node in reach gathers node by node, and the host does not see the mask (the
+    // autotuner times it).  So untuned it is taken only where no mask measured (a square; 1, 10
+    // and 40 % of the nodes at random) makes it the slower one by more than 3 %.
+    // us a step on GB300, square / 10 %, the register kernel in brackets: D2Q9 FP64 64^2
+    // 7.3 (11) / 7.8 (13), 512^2 48 (55) / 54 (57), D3Q19 FP64 128^3 691 (704) / 718
+    // (708), D2Q9 FP16 2048^2 49 (108) / 156 (182).  Elsewhere it loses up to threefold:
+    // D2Q9 FP32 128 x 4096 36 (20) / 54 (25), 2048^2 83 (94) / 172 (129), D3Q19 FP32
+    // 128^3 181 (142) / 308 (178), D3Q27 FP64 64^3 250 (216) / 290 (218).
+    // One node per thread on small lattices and short 16-bit rows, which wider threads leave
+    // with too few warps, and on D3Q27, against the widest: D2Q9 FP32 64^2 4.9 (7.9) / 5.5
+    // (9.2), 320^2 6.4 (8.6) / 6.6 (10), but 1024^2 29 (23) / 32 (30); FP16 64 x 65536 140
+    // (630) / 158 (725); D3Q19 FP32 48^3 13 (23), but 128^3 156 (142); D3Q27 FP32 192^3
+    // 900 (1295) / 955 (1513).
+    const bool half9 = pl.Q == 9 && pl.esize == 2;
+    const bool one = pl.Q == 27 || pl.N <= (1LL << 17) || (half9 && pl.p.nx < 256);
+    if ((pl.esize == 8 && pl.Q != 27) || (half9 && !one))
+      for (size_t k = 0; k < vs.size(); ++k)
+        if (vs[k].kind == 1 && vs[k].bx == 0 && (pl.Q == 9 || vs[k].stages == 2)) return (int)k;
+    return default_register(pl, vs, one ? 1 : 8);
+  }
   // 16-bit storage, A/B: four nodes per thread (D2Q9 2048^2 27 us a step against 31
   // with two, 4096^2 96 / 111; D3Q19 256^3 273 / 504, 96^3 38 / 70).
   const bool aa = pl.p.layout == LBM_LAYOUT_AA;
@@ -220,24 +258,13 @@ static int default_single(const Plan& pl, const std::vector<Variant>& vs) {
       for (size_t k = 0; k < vs.size(); ++k)
         if (vs[k].kind == 0 && vs[k].nv == 1 && vs[k].bx == 32 && vs[k].by == 8) return (int)k;
   }
-  // the pipelined kernel when available, else the widest vector that keeps the
-  // registers of one thread moderate, 256 threads
+  // the pipelined kernel when available, else a register kernel
   for (size_t k = 0; k < vs.size(); ++k)
     if (vs[k].kind == 1) return (int)k;
-  const int budget = pl.Q == 9 ? 16 : 8;  // bytes per plane per thread
-  int best = 0, best_nv = 0;
-  for (size_t k = 0; k < vs.size(); ++k) {
-    const Variant& v = vs[k];
-    if (v.kind != 0 || v.nv * pl.esize > budget || v.bx * v.by != 256) continue;
-    if (v.nv > best_nv || (v.nv == best_nv && v.bx == 64)) {
-      best = (int)k;
-      best_nv = v.nv;
-    }
-  }
-  return best;
+  return default_register(pl, vs, 8);
 }
 
-int default_variant(const Plan& pl, const std::vector<Variant>& vs) {
+int default_variant(const Plan& pl, const std::vector<Variant>& vs, bool masked) {
   // Two steps per launch where they are available: they beat the fastest
   // single-step variant on every size measured (us per step, GB300; FP32: 64^2
   // 2.4 / 3.2, 1024^2 8.6 / 10.7, 2048^2 27 / 48, 4096^2 98 / 183, 64 x 65536 70 / 131;
@@ -250,7 +277,7 @@ int default_variant(const Plan& pl, const std::vector<Variant>& vs) {
   const bool bound = pl.esize == 2 && pl.p.nx % 8 == 0 && pl.N >= (1LL << 20);
   for (size_t k = 0; k < vs.size(); ++k)
     if (!bound && vs[k].kind == 2 && vs[k].X == (pl.p.nx <= 256 ? 256 : 512)) return (int)k;
-  return default_single(pl, vs);
+  return default_single(pl, vs, masked);
 }
 
 }  // namespace lbm
@@ -335,7 +362,7 @@ StepLaunch step_of(lbm_ctx* c, const Variant& v) {
 // or the default of single steps where `var` takes two steps per launch.
 static int single_variant(const Plan& pl, const std::vector<Variant>& vs, int var) {
   if (vs[var].kind != 2) return var;
-  return default_single(pl, vs);
+  return default_single(pl, vs, false);  // (no mask with two steps per launch)
 }
 
 int ctx_new(const Plan& pl, cudaStream_t st, lbm_ctx** out) {
@@ -347,7 +374,7 @@ int ctx_new(const Plan& pl, cudaStream_t st, lbm_ctx** out) {
   cudaGetDevice(&c->device);
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   c->vars = variants_for(pl, c->ops, false);
-  c->var = default_variant(pl, c->vars);
+  c->var = default_variant(pl, c->vars, false);
   c->var_one = single_variant(c->pl, c->vars, c->var);
   *out = c;
   return LBM_OK;
@@ -363,7 +390,7 @@ int ctx_bind(lbm_ctx* c, void* a, void* b, const uint8_t* mask, void* scratch) {
   c->cur = 0;
   c->t = 0;
   c->vars = variants_for(c->pl, c->ops, mask != nullptr);
-  c->var = default_variant(c->pl, c->vars);
+  c->var = default_variant(c->pl, c->vars, mask != nullptr);
   c->var_one = single_variant(c->pl, c->vars, c->var);
   c->var_odd = -1;
   return LBM_OK;

@@ -34,7 +34,7 @@ struct Plan {
 
 int plan(const lbm_params* p, Plan* out);
 std::vector<Variant> variants_for(const Plan& pl, const Ops* ops, bool masked);
-int default_variant(const Plan& pl, const std::vector<Variant>& vs);
+int default_variant(const Plan& pl, const std::vector<Variant>& vs, bool masked);
 
 int ctx_new(const Plan& pl, cudaStream_t st, lbm_ctx** out);
 int ctx_bind(lbm_ctx* c, void* a, void* b, const uint8_t* mask, void* scratch);
