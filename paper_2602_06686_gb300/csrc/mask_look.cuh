@@ -11,13 +11,14 @@ namespace lbm {
 __host__ __device__ constexpr int mask_column(int x, int nx) { return x < nx ? x : nx - 1; }
 
 // The column beside the warp's 32 consecutive nodes: lane 0 (the first) looks to
-// the left, lane 31 to the right, with the wrap of a periodic row; other lanes
-// have none and repeat their own.  A lane 31 at or beyond the row's last node looks
+// the left of its own, lane 31 to the right, with the wrap of a periodic row; other
+// lanes have none and repeat their own.  A lane 31 at or beyond the row's last node looks
 // at column 0, so that the wrapped neighbour of a last node in mid-warp is seen.
 __host__ __device__ constexpr int mask_column_beside(int x, int nx, int lane) {
-  return lane == 0    ? (x == 0 ? nx - 1 : mask_column(x - 1, nx))
-         : lane == 31 ? (x >= nx - 1 ? 0 : x + 1)
-                      : mask_column(x, nx);
+  const int c = mask_column(x, nx);
+  return lane == 0    ? (c == 0 ? nx - 1 : c - 1)
+         : lane == 31 ? (c == nx - 1 ? 0 : c + 1)
+                      : c;
 }
 
 }  // namespace lbm

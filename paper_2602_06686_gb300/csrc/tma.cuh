@@ -713,13 +713,10 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
     const int wdt = min(XT, G.nx - x0);
     bool near = false;  // MODE 5: a solid node is in reach of this warp's nodes
     if constexpr (MODE == 5) {
-      // before the wait for the stage, so that the mask's latency overlaps the copy's;
-      // a warp beyond the row's end has no node to look around
-      if (__any_sync(0xffffffffu, jn[0] < wdt)) {
-        near = mask_near<L>(G, a.mask, x0 + jn[0], y, z, ADJ ? 0 : lane);
-        if (PACK) near |= mask_near<L>(G, a.mask, x0 + jn[NPT - 1], y, z, ADJ ? 31 : lane);
-        near = __any_sync(0xffffffffu, near);
-      }
+      // before the wait for the stage, so that the mask's latency overlaps the copy's
+      near = mask_near<L>(G, a.mask, x0 + jn[0], y, z, ADJ ? 0 : lane);
+      if (PACK) near |= mask_near<L>(G, a.mask, x0 + jn[NPT - 1], y, z, ADJ ? 31 : lane);
+      near = __any_sync(0xffffffffu, near);
     }
     if (!mbar_wait_warp(smem_addr(full + s), u & 1u, abort_flag, a.err, a.timeout_ns)) break;
     const T* st = reinterpret_cast<const T*>(ringb + s * stage_bytes);
