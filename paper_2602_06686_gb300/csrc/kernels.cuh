@@ -49,14 +49,23 @@ struct StepArgs {
 // Programmatic dependent launch between consecutive update kernels of a stream
 // (launch_chained): the next launch's blocks are placed while this one runs and
 // wait here until it has completed and its writes are visible.  Every thread of
-// a chained kernel calls it before it touches global memory.  A value that every
-// address depends on passes through, so that no load (read-only path included)
-// can move above the wait: the base pointer in the pipelined kernels, which
-// hold it in a register anyway, and the node's x in the one-pass kernels, whose
-// base pointers stay kernel parameters (passing the pointer through there costs
-// 4 to 8 registers: D2Q9 FP16 four nodes per thread 64 -> 72, 3 % of a
-// 2250 x 1410 step; FP32 with a mask 6 % of a 2048 x 1024 step).  A launch lets its successor start once it has passed its own wait, so
-// at most one launch waits behind a running one.
+// a chained kernel calls it before it touches global memory.  A launch lets its
+// successor start once it has passed its own wait, so at most one launch waits behind
+// a running one.
+//
+// The clobber keeps ordinary loads and stores below the wait; a load that the compiler may
+// send down the read-only path needs an address that depends on it.  So a value passes
+// through that such addresses are formed from, chosen by what it costs:
+//  * the one-pass kernels: the node's x, or threadIdx.x.  Their base pointers stay kernel
+//    parameters, since a pointer that passes through costs 4 to 8 registers (D2Q9 FP16
+//    four nodes per thread 64 -> 72, 3 % of a 2250 x 1410 step; FP32 with a mask 6 % of a
+//    2048 x 1024 step);
+//  * k_step_tma and k_step_pair: the source pointer, which few consumers read (with
+//    threadIdx.x instead D3Q19 FP16 takes 235 us a step of a 512 x 64 x 512 channel
+//    against 233), and the consumer's index where a solid mask is read;
+//  * k_step_aa_tma reads and writes one buffer, so none of its loads is read-only: the
+//    buffer stays a parameter and its accesses global ones, not generic (D3Q19 FP16
+//    208^3 538 us a step against 543).
 template <typename P>
 __device__ __forceinline__ P* chain_wait(P* p) {
   asm volatile("griddepcontrol.wait;" : "+l"(p)::"memory");
@@ -66,6 +75,12 @@ __device__ __forceinline__ P* chain_wait(P* p) {
 __device__ __forceinline__ int chain_wait(int x) {
   asm volatile("griddepcontrol.wait;" : "+r"(x)::"memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  return x;
+}
+
+// Another value that addresses are formed from, behind a chain_wait that has been passed.
+__device__ __forceinline__ int behind_wait(int x) {
+  asm volatile("" : "+r"(x)::"memory");
   return x;
 }
 

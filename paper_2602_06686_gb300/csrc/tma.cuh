@@ -699,7 +699,8 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
   // 32-bit storage keeps the split pair (x0 + j, x0 + j + X/2), whose scalar
   // shared reads are free of bank conflicts for every x shift.
   constexpr bool ADJ = PACK && sizeof(T) == 2;
-  const int ct = threadIdx.x - Sh::kBase;  // 0 .. kConsumers-1: this thread's node (pair)
+  int ct = threadIdx.x - Sh::kBase;  // 0 .. kConsumers-1: this thread's node (pair)
+  if constexpr (MODE == 5) ct = behind_wait(ct);  // the mask's addresses are formed from it
   int jn[NPT];
   jn[0] = ADJ ? 2 * ct : ct;
   if (PACK) jn[NPT - 1] = ADJ ? 2 * ct + 1 : ct + XT / 2;
