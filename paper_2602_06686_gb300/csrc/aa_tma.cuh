@@ -224,6 +224,12 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, ODD ? 1 : 0>::kThreads,
   int jn[NPT];
   jn[0] = ADJ ? 2 * ct : ct;
   if (PACK) jn[NPT - 1] = ADJ ? 2 * ct + 1 : ct + XT / 2;
+  if constexpr (!ODD && ADJ) {
+    if (G.nx <= XT && jn[0] - 2 * lane >= G.nx) {
+      idle_consumer(a.ntiles, G.ny, ST, full, empty, abort_flag, a.err, a.timeout_ns);
+      return;
+    }
+  }
   TileWalk w(a.ntiles, a.ntx, G.ny);
   int s = 0;
   uint32_t u = 0;
@@ -242,10 +248,10 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, ODD ? 1 : 0>::kThreads,
     bool act[NPT];
 #pragma unroll
     for (int n = 0; n < NPT; ++n) act[n] = jn[n] < wdt;
-    if constexpr (!ODD) {  // (the odd step's staging counts every warp)
+    if constexpr (!ODD && !ADJ) {  // (the odd step's staging counts every warp)
       // a warp beyond the row's end has no node in this tile: it releases the
-      // stage and spends no arithmetic on it
-      if (__all_sync(0xffffffffu, !act[0])) {
+      // stage and spends no arithmetic on it (a full tile does not vote)
+      if (wdt < XT && __all_sync(0xffffffffu, !act[0])) {
         if (lane == 0) mbar_arrive(smem_addr(empty + s));
         if (++s == ST) {
           s = 0;

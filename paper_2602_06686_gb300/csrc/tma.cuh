@@ -212,6 +212,28 @@ struct TileWalk {
   }
 };
 
+// A consumer warp without a node in any tile, where a tile holds a whole row that ends
+// before the warp: it takes part in the stages' barriers and spends no arithmetic.  The
+// kernels bound by 16-bit arithmetic sort such warps out here, ahead of everything
+// else, since a test in the tile loop costs every warp of a full tile (D3Q19 FP16, four nodes
+// per thread, 512-wide tiles: a 512 x 64 x 512 channel 230 us a step, with the test in the
+// loop 233; but a 96^3 lattice 39 instead of 45 with idle warps that compute).
+__device__ __forceinline__ void idle_consumer(int ntiles, int ny, int stages, uint64_t* full,
+                                              uint64_t* empty, volatile int* abort_flag, int* err,
+                                              long long timeout_ns) {
+  TileWalk w(ntiles, 1, ny);  // one tile a row
+  int s = 0;
+  uint32_t u = 0;
+  for (; w.more(); w.next()) {
+    if (!mbar_wait_warp(smem_addr(full + s), u & 1u, abort_flag, err, timeout_ns)) break;
+    if ((threadIdx.x & 31) == 0) mbar_arrive(smem_addr(empty + s));
+    if (++s == stages) {
+      s = 0;
+      ++u;
+    }
+  }
+}
+
 template <class L>
 __device__ __forceinline__ int opp_dyn(int i) {
   int r = 0;
@@ -430,6 +452,11 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
   const T* __restrict__ src = static_cast<const T*>(chain_wait(a.src));
   T* __restrict__ dst = static_cast<T*>(a.dst);
 
+  if (MODE == 4 && warp > 0 && G.nx <= XT && 128 * (warp - 1) >= G.nx) {
+    idle_consumer(a.ntiles, G.ny, ST, full, empty, abort_flag, a.err, a.timeout_ns);
+    return;
+  }
+
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     // Lane i (< Q) copies population plane i; lane 0 sets the expected byte
@@ -604,16 +631,6 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
       bool act[4];
 #pragma unroll
       for (int n = 0; n < 4; ++n) act[n] = j0 + n < wdt;
-      // a warp beyond the row's end has no node in this tile: it releases the
-      // stage and spends no arithmetic on it
-      if (__all_sync(0xffffffffu, !act[0])) {
-        if (lane == 0) mbar_arrive(smem_addr(empty + s));
-        if (++s == ST) {
-          s = 0;
-          ++u;
-        }
-        continue;
-      }
       F2 ga[L::Q], gb[L::Q];
       if (!anywall && !xwall) {
 #pragma unroll
@@ -733,8 +750,9 @@ __global__ void __launch_bounds__(TmaShape<XT, PACK, MODE == 3 ? 1 : 0, MODE == 
     for (int n = 0; n < NPT; ++n) act[n] = jn[n] < wdt;
     if constexpr (MODE != 3) {
       // a warp beyond the row's end has no node in this tile: it releases the
-      // stage and spends no arithmetic on it
-      if (__all_sync(0xffffffffu, !act[0])) {
+      // stage and spends no arithmetic on it (only a ragged tile has such a warp, so
+      // a full one does not vote)
+      if (wdt < XT && __all_sync(0xffffffffu, !act[0])) {
         if (lane == 0) mbar_arrive(smem_addr(empty + s));
         if (++s == ST) {
           s = 0;
