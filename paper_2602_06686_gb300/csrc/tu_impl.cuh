@@ -594,8 +594,8 @@ __global__ void __launch_bounds__(256) k_momentum(Geo G, const uint8_t* mask, in
 // takes 3.1 us a step on 64^2 and 5.4 us on 512^2, plain launches take 6.2 us
 // and 8.2 us; from 2048^2 on the two are equal within 2 %.
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
-                                  cudaStream_t st, A&&... args) {
+inline cudaError_t launch_update(bool chained, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                                 cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -605,8 +605,13 @@ inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, siz
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = chained ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t st, A&&... args) {
+  return launch_update(true, kern, grid, block, smem, st, args...);
 }
 
 // Resident blocks per SM of a kernel with `smem` bytes of dynamic shared memory on the
@@ -755,7 +760,19 @@ struct TU {
     const int resident = s.v.bx > 0 && s.v.bx < per_sm ? s.v.bx : per_sm;
     long long blocks = (long long)resident * (s.sms > 0 ? s.sms : 1);
     if (blocks > a.ntiles) blocks = a.ntiles;
-    return launch_chained(kern, dim3((unsigned)blocks), dim3(threads), smem, s.stream, a);
+    // Chained only where the blocks of two launches fit on the chip together, if the step
+    // depends on how many blocks an SM holds: with a capped number (bx), and for
+    // D2Q9 in FP64, whose short tiles are bound by the SM's pipe.  Otherwise the next launch's
+    // blocks take slots as this one's fall free, three on one SM and none on another, and the
+    // step waits for the fullest SM.  us a step, chained / not: D2Q9 FP32 4096^2 with walls,
+    // two blocks an SM 192 / 184; FP64 TRT-RLB 224^2 20 / 23, 240^2 32 / 25, 512^2 88 / 74,
+    // P-TRT 256^2 20 / 16, 512^2 55 / 47; the gain given up elsewhere is at most a tenth
+    // (320^2 26 / 29) and nothing from 1000^2 on.  In place the two parities hold
+    // different numbers of blocks, and one block an SM is the line (TRT-RLB 128^2 12.9 /
+    // 13.3, 208^2 25.9 / 24.6).
+    const bool room = kind == 1 || kind == 2 ? blocks <= s.sms : 2 * blocks <= (long long)per_sm * s.sms;
+    const bool chained = room || !(resident < per_sm || (L::Q == 9 && sizeof(R) == 8));
+    return launch_update(chained, kern, dim3((unsigned)blocks), dim3(threads), smem, s.stream, a);
   }
 
   template <int COLL, bool FORCE>
