@@ -249,10 +249,17 @@ static int default_single(const Plan& pl, const std::vector<Variant>& vs, bool m
     // Rows that fill too little of a tile are better off in the register kernel
     // (D3Q19 FP32 64^3 14.5 us against 23.5, 32^3 5.5 / 8.5, 128^3 109 / 90; AA 160^3, a tile of
     // 256: 173 / 192; FP16 96^3 49 / 38).  FP64 is bound by its pipe either way.
-    const bool narrow = pl.esize == 8 ? false
-                        : aa          ? 3 * pl.p.nx < 2 * best_pad
-                        : quad        ? pl.p.nx < 96
-                                      : pl.p.nx < 128;
+    // But where every block has one tile, or two, the register kernel's longer chain of
+    // loads is all that counts (up to four rows an SM, pipeline / register: D3Q27 FP16
+    // 64 x 16^2 6.3 / 13, 24^3 6.5 / 12, FP32 24^3 7.9 / 9.6, D3Q19 FP16 64 x 16^2 4.7 / 8.7,
+    // 24^3 5.0 / 8.4; beyond, D3Q27 FP16 32^3 8.7 / 9.9 and with walls 9.9 / 9.9, 16 x 64^2
+    // 24 / 14).  D3Q19 FP32 gains nothing at 24^3 (6.4 / 6.5) and stays as it is.
+    const long long rows = (long long)pl.p.ny * pl.p.nz;
+    const bool few = !aa && rows <= 608 && (pl.Q == 27 || (quad && rows >= 32));
+    const bool narrow = pl.esize == 8 || few ? false
+                        : aa                 ? 3 * pl.p.nx < 2 * best_pad
+                        : quad               ? pl.p.nx < 96
+                                             : pl.p.nx < 128;
     if (best >= 0 && !narrow) return best;
     if (best >= 0)
       for (size_t k = 0; k < vs.size(); ++k)
