@@ -320,7 +320,9 @@ const char* lbm_last_error(void);
  * another for the odd steps (lbm_get_variant reports the even steps' one).
  * Variants named tma2_* take two steps per launch: lbm_step(n) runs 2 (n / 4) such
  * launches and the rest of the n steps singly, so that the state is in the same
- * buffer as after n single steps, and the bits of the state are the same. */
+ * buffer as after n single steps.  Its values are the same too: the same bits as the
+ * single steps of the other tma_* variants, and up to the sign of a zero those of
+ * the nv* variants, which add a zero force where there is none. */
 int lbm_variant_count(const lbm_ctx* ctx, int* n);
 int lbm_variant_name(const lbm_ctx* ctx, int v, char* buf, size_t len);
 int lbm_get_variant(const lbm_ctx* ctx, int* v);

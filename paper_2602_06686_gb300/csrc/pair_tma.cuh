@@ -30,7 +30,8 @@
 //
 // Both steps run the collision of the single-step kernel in the same order and
 // round the intermediate state to the storage type, so the results are the
-// same bits as two single steps.
+// same bits as two single steps of the pipelined kernel (up to the sign of a zero those
+// of the register kernels, which add a zero force where there is none).
 //
 // Every wait is bounded as in k_step_tma.  A warp whose wait ran out stays in
 // the row loop and only arrives at the block barriers, so no warp is left
