@@ -876,15 +876,18 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
   const bool aa = c->pl.p.layout == LBM_LAYOUT_AA;
   // Everything that a candidate's kernel or time depends on.  With open boundaries all of them
   // run the same kernel, and with a force another instantiation.
-  using Key = std::array<int, 15>;
+  using Key = std::array<int, 14>;
   static std::mutex mu;
   // variant, AA odd-step variant or -1, variant of single steps
   static std::map<Key, std::tuple<int, int, int>> cache;
-  const Key key{c->pl.p.lattice, c->pl.p.storage, c->pl.kernel_collision, c->mask != nullptr,
-                c->pl.p.nx,      c->pl.p.ny,      c->pl.p.nz,            c->pl.g.per[0],
-                c->pl.g.per[1],  c->pl.g.per[2],  c->pl.p.layout,        c->scheme,
-                c->open.on,      c->pl.force,     c->device};
-  if (!times_ms) {
+  const Key key{c->pl.p.lattice, c->pl.p.storage, c->pl.kernel_collision, c->pl.p.nx,
+                c->pl.p.ny,      c->pl.p.nz,      c->pl.g.per[0],         c->pl.g.per[1],
+                c->pl.g.per[2],  c->pl.p.layout,  c->scheme,              c->open.on,
+                c->pl.force,     c->device};
+  // With a solid mask the times depend on where the solid nodes lie, which the key does not say:
+  // every such lattice is timed (a square and 10 % of the nodes at random want different kernels).
+  const bool keep_choice = c->mask == nullptr;
+  if (!times_ms && keep_choice) {
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
     if (it != cache.end() && std::get<0>(it->second) < (int)c->vars.size() &&
@@ -995,7 +998,7 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
   }
   c->var = best;
   c->var_one = c->vars[best].kind == 2 ? best_one : best;
-  {
+  if (keep_choice) {
     std::lock_guard<std::mutex> lk(mu);
     cache[key] = std::make_tuple(best, c->var_odd, c->var_one);
   }
