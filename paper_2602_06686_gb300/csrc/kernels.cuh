@@ -56,7 +56,10 @@ struct StepArgs {
 // The clobber keeps ordinary loads and stores below the wait; a load that the compiler may
 // send down the read-only path needs an address that depends on it.  So a value passes
 // through that such addresses are formed from, chosen by what it costs:
-//  * the one-pass kernels: the node's x, or threadIdx.x.  Their base pointers stay kernel
+//  * the one-pass kernels: the node's x, threadIdx.x or blockIdx.x, whichever costs no register
+//    (k_step_ab without a mask: blockIdx.x; D3Q19 FP16 TRT-RLB one node per thread 55, with x
+//    57, which leaves an SM one block less: 150 x 131 x 117 187 us a step against 174; with
+//    a mask blockIdx.x makes eight nodes per thread spill).  Their base pointers stay kernel
 //    parameters, since a pointer that passes through costs 4 to 8 registers (D2Q9 FP16
 //    four nodes per thread 64 -> 72, 3 % of a 2250 x 1410 step; FP32 with a mask 6 % of a
 //    2048 x 1024 step);
@@ -260,7 +263,8 @@ __device__ __forceinline__ void update_chunk(const StepArgs<typename S::R>& a, i
 template <class L, int COLL, class S, int NV, bool MASK>
 __global__ void __launch_bounds__(256) k_step_ab(const StepArgs<typename S::R> a) {
   const int lane = threadIdx.x & 31;
-  const int x0 = chain_wait((int)(blockIdx.x * blockDim.x + threadIdx.x)) * NV;
+  const int x0 = (MASK ? chain_wait((int)(blockIdx.x * blockDim.x + threadIdx.x))
+                       : (int)(chain_wait((int)blockIdx.x) * blockDim.x + threadIdx.x)) * NV;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
   if (y >= a.g.ny) return;  // whole warps (blockDim.x is a multiple of 32)
