@@ -226,16 +226,20 @@ __global__ void __launch_bounds__(256) k_step_s2_aa(const StepArgs<typename S::R
   const RowNode q(G, chain_wait((int)threadIdx.x));
   if (!q.valid || (a.mask && a.mask[q.n])) return;
   T* buf = static_cast<T*>(a.dst);
-  // the differences first: phi is no read-only array (the launch before this one writes it
-  // while blocks of this one wait), so its loads keep their place, and behind the
-  // populations' they add ten registers (D3Q27 FP16 96^3 187 us a step, this order 171)
-  R Dg[3] = {R(0), R(0), R(0)};
+  R g[L::Q], Dg[3] = {R(0), R(0), R(0)};
+  const auto differences = [&] {
 #pragma unroll
-  for (int d = 0; d < L::D; ++d) Dg[d] = phi_grad<L, R>(G, a.mask, phi, d, q.x, q.y, q.z, q.n);
-  R g[L::Q];
+    for (int d = 0; d < L::D; ++d) Dg[d] = phi_grad<L, R>(G, a.mask, phi, d, q.x, q.y, q.z, q.n);
+  };
+  // In three dimensions the differences first: phi is no read-only array (the launch before
+  // this one writes it while blocks of this one wait), so its loads keep their place, and
+  // behind the populations' they add ten registers (D3Q27 FP16 96^3 187 us a step, this order
+  // 171; D3Q19 FP32 128^3 240 / 237; but D2Q9 FP32 2048^2 176 / 189).
+  if (L::D == 3) differences();
 #pragma unroll
   for (int i = 0; i < L::Q; ++i)
     g[i] = S::dec(buf[aa_state_slot<L>(G, a.mask, parity, q.x, q.y, q.z, i)]);
+  if (L::D != 3) differences();
   const bool bad = collide_v<L, COLL, FORCE, R>(g, a.c) != 0u;
   const R third = (Dg[0] + Dg[1] + Dg[2]) * R(1.0 / 3.0);
   const long long own = ((long long)q.z * G.ny + q.y) * G.pitch + q.x;
