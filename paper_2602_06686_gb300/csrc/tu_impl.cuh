@@ -773,9 +773,13 @@ struct TU {
     // P-TRT 256^2 20 / 16, 512^2 55 / 47; the gain given up elsewhere is at most a tenth
     // (320^2 26 / 29) and nothing from 1000^2 on.  In place the two parities hold
     // different numbers of blocks, and one block an SM is the line (TRT-RLB 128^2 12.9 /
-    // 13.3, 208^2 25.9 / 24.6).
-    const bool room = kind == 1 || kind == 2 ? blocks <= s.sms : 2 * blocks <= (long long)per_sm * s.sms;
-    const bool chained = room || !(resident < per_sm || (L::Q == 9 && sizeof(R) == 8));
+    // 13.3, 208^2 25.9 / 24.6); there it holds for 16-bit storage in three dimensions too
+    // (untuned D3Q19 FP16 160^3 321 / 297, D3Q27 192^3 526 / 511, 384-wide tiles 551 / 386).
+    const bool inplace = kind == 1 || kind == 2;
+    const bool room = inplace ? blocks <= s.sms : 2 * blocks <= (long long)per_sm * s.sms;
+    const bool uneven = resident < per_sm || (L::Q == 9 && sizeof(R) == 8) ||
+                        (inplace && L::D == 3 && sizeof(T) == 2);
+    const bool chained = room || !uneven;
     return launch_update(chained, kern, dim3((unsigned)blocks), dim3(threads), smem, s.stream, a);
   }
 

@@ -10,16 +10,19 @@ from gpu_cases import gpu_lattice
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("ny,storage,layout", [
-    (228, "F64", "AB"), (229, "F64", "AB"),  # two launches of three blocks an SM fit, or not
-    (152, "F64", "AA"), (153, "F64", "AA"),  # in place: one block an SM
-    (600, "F32", "AB"),                      # with a capped number of blocks
+@pytest.mark.parametrize("lat,shape,storage,layout", [
+    (O.D2Q9, (1, 228, 24), "F64", "AB"),    # two launches of three blocks an SM fit
+    (O.D2Q9, (1, 229, 24), "F64", "AB"),    # or not
+    (O.D2Q9, (1, 152, 24), "F64", "AA"),    # in place: one block an SM
+    (O.D2Q9, (1, 153, 24), "F64", "AA"),
+    (O.D2Q9, (1, 600, 24), "F32", "AB"),    # with a capped number of blocks
+    (O.D3Q19, (12, 12, 24), "F16", "AA"),   # 144 rows
+    (O.D3Q19, (12, 14, 24), "BF16", "AA"),  # 168
 ])
-def test_chained_and_plain_launches_give_one_state(ny, storage, layout):
+def test_chained_and_plain_launches_give_one_state(lat, shape, storage, layout):
     rng = np.random.default_rng(67)
-    shape = (1, ny, 24)
-    rho, u = W.random_macros(shape, 2, rng, umax=0.05)
-    g = gpu_lattice(O.D2Q9, shape, O.TRT_RLB, 0.03, 0.25, storage=storage, layout=layout,
+    rho, u = W.random_macros(shape, O.D_OF[lat], rng, umax=0.05)
+    g = gpu_lattice(lat, shape, O.TRT_RLB, 0.03, 0.25, storage=storage, layout=layout,
                     force=(1e-5, 0.0, 0.0), periodic=(1, 0, 1))
     names = g.variants()
     out = {}
