@@ -337,8 +337,10 @@ int lbm_set_variant(lbm_ctx* ctx, int v);
  * 2 (reps + 1) or 2 reps + 3 steps per variant and the step counter with it;
  * the even and odd steps are different kernels and each gets its own fastest
  * variant (times_ms then holds the mean of the two per variant).  Results are
- * cached per (lattice, storage, collision, mask, extent, layout, forcing
- * scheme) for the process; a cached answer (times_ms NULL) runs nothing.
+ * cached per (lattice, storage, collision, mask or none, extent, layout, forcing
+ * scheme, open boundaries, force or none, device) for the process; a cached
+ * answer (times_ms NULL) runs nothing.  A/B lattices with a solid mask are
+ * timed at every call, since their best kernel depends on the mask itself.
  * Under forcing scheme 2 the trials are scheme-2 steps.  Synchronises. */
 int lbm_autotune(lbm_ctx* ctx, int reps, int* chosen, float* times_ms);
 

@@ -876,17 +876,19 @@ int lbm_autotune(lbm_ctx* c, int reps, int* chosen, float* times_ms) {
   const bool aa = c->pl.p.layout == LBM_LAYOUT_AA;
   // Everything that a candidate's kernel or time depends on.  With open boundaries all of them
   // run the same kernel, and with a force another instantiation.
-  using Key = std::array<int, 14>;
+  using Key = std::array<int, 15>;
   static std::mutex mu;
   // variant, AA odd-step variant or -1, variant of single steps
   static std::map<Key, std::tuple<int, int, int>> cache;
-  const Key key{c->pl.p.lattice, c->pl.p.storage, c->pl.kernel_collision, c->pl.p.nx,
-                c->pl.p.ny,      c->pl.p.nz,      c->pl.g.per[0],         c->pl.g.per[1],
-                c->pl.g.per[2],  c->pl.p.layout,  c->scheme,              c->open.on,
-                c->pl.force,     c->device};
-  // With a solid mask the times depend on where the solid nodes lie, which the key does not say:
-  // every such lattice is timed (a square and 10 % of the nodes at random want different kernels).
-  const bool keep_choice = c->mask == nullptr;
+  const Key key{c->pl.p.lattice, c->pl.p.storage, c->pl.kernel_collision, c->mask != nullptr,
+                c->pl.p.nx,      c->pl.p.ny,      c->pl.p.nz,            c->pl.g.per[0],
+                c->pl.g.per[1],  c->pl.g.per[2],  c->pl.p.layout,        c->scheme,
+                c->open.on,      c->pl.force,     c->device};
+  // On a masked A/B lattice the best kernel depends on where the solid nodes lie, which the key
+  // does not say, so each is timed (a square and 10 % of the nodes at random want different
+  // kernels).  In place the masked candidates are register kernels alone, whose order depends
+  // little on the mask, and a trial advances the lattice: there the choice is remembered.
+  const bool keep_choice = c->mask == nullptr || aa;
   if (!times_ms && keep_choice) {
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
