@@ -42,12 +42,11 @@ BYTES_PER_NODE = {("D2Q9", "F64"): 144, ("D2Q9", "F32"): 72, ("D2Q9", "F16"): 36
                   ("D3Q27", "F32"): 216, ("D3Q27", "F16"): 108, ("D3Q27", "BF16"): 108}
 PROFILE = os.path.join(ROOT, "profiles", "stream_collide_d2q9_f32_4096.md")
 # FP64 instructions (DADD + DMUL + DFMA) per node update of the FP64 update, by
-# lattice and collision.  TRT-RLB: ncu counts on D3Q19 128^3 and D2Q9 2048x1024
-# (profiles/stream_collide_d3q19_f64_128.md).  P-TRT and TRT: counted from the
-# moment-space form in collide_v.cuh, with 7 for the reciprocal.  With GB300's 2
-# FP64 lanes per SM they give the FP64-pipe roofline of the FP64 runs.
-FP64_INSTR_PER_NODE = {("D3Q19", "P_TRT"): 162, ("D3Q19", "TRT_RLB"): 301, ("D3Q19", "TRT"): 166,
-                       ("D2Q9", "P_TRT"): 80, ("D2Q9", "TRT_RLB"): 129, ("D2Q9", "TRT"): 82}
+# lattice and collision: ncu counts on D3Q19 128^3 and D2Q9 2048x1024
+# (profiles/stream_collide_d3q19_f64_128.md).  With GB300's 2 FP64 lanes per
+# SM they give the FP64-pipe roofline of the FP64 runs.
+FP64_INSTR_PER_NODE = {("D3Q19", "P_TRT"): 159, ("D3Q19", "TRT_RLB"): 301, ("D3Q19", "TRT"): 157,
+                       ("D2Q9", "P_TRT"): 77, ("D2Q9", "TRT_RLB"): 129, ("D2Q9", "TRT"): 77}
 FP64_LANES_PER_SM = 2
 
 
